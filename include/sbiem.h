@@ -491,7 +491,11 @@ int sbiem_footprint(sbiem_t s, int64_t* history_bytes_per_step, int64_t* device_
  *   shape: lags per chunk x stages in flight; the chunk length is fixed at
  *     creation (shape 3: 2048 lags FP32, 1024 FP64, two stages), so only
  *     shapes of that chunk length are accepted (0 and 2, or 1, or 3 and 4;
- *     shape 4 is shape 3's chunk in one stage).
+ *     shape 4 is shape 3's chunk in one stage).  In FP64, in FP32 above N =
+ *     16384 and in ensembles shape 3 is the direct sweep instead: one warp
+ *     per run of lags, ring slots loaded into registers, no staging in shared
+ *     memory and so no copy waits (a handle with a wait limit of its own
+ *     sweeps in the bulk-async form).
  *   gen_ds_max (FP32 form only): where the weights come from.  The
  *     midpoint weights w_{n,j} = dt_min C(s) at s = (j + 1/2) ds_n,
  *     ds_n = c_s k_n dt_min, depend on the mode only through ds_n; modes
@@ -504,7 +508,9 @@ int sbiem_footprint(sbiem_t s, int64_t* history_bytes_per_step, int64_t* device_
  *     materialized weights with the slots.  0 streams every mode's weights;
  *     modes with ds up to 1/64 evaluate in blocks of eight lags, modes
  *     above it (up to 1/32, the largest step a four-lag block allows;
- *     larger values are taken as 1/32) in blocks of four.  1/64 is the
+ *     larger values are taken as 1/32) in blocks of four.  The direct sweep
+ *     evaluates lag by lag from a table of its own: any value above 0 puts
+ *     every mode's weights on chip.  1/64 is the
  *     default of a new FP32 handle whenever its windows' s range fits the
  *     table (k_c L <= about 340 rad); table_err is the
  *     table's largest error relative to dt_min max|C| (-1: no table).

@@ -25,7 +25,8 @@ namespace {
 
 thread_local std::string g_last_error;
 
-// Sweep shape of a new handle (chunk length x stages in flight).
+// Sweep shape of a new handle (chunk length x stages in flight; the direct
+// sweep where direct_form says so).
 constexpr int kDefaultSweepShape = 3;
 // Largest on-chip weight table (bytes): it is read through L1 beside the
 // sweep's stages in shared memory.
@@ -112,6 +113,10 @@ struct sbiem_s {
   int gen_pieces = 0;   // pieces of the on-chip weight table (0: none, weights streamed)
   float gen_ds_max = 0;  // modes with ds = c_s k_n dt_min <= this evaluate their weights on chip
   double gen_err = 0.0; // its largest error relative to dt max|C|
+  // direct sweep: its weight table (NULL: the weights are streamed) and error
+  const float4* direct_wtab = nullptr;
+  int direct_pieces = 0;
+  double direct_err = 0.0;
   // timing probe: 4 events per slot; graph event-record nodes are retargeted
   // to the slot of each launch
   int pslots = 0;
@@ -245,20 +250,111 @@ void windows(const sbiem_params& p, double L, double dt_min, std::vector<int64_t
   for (size_t n = 0; n < MT.size(); ++n) M[n] = std::max(MT[n], MN[n]);
 }
 
+// Whether a handle's sweep of this shape is the direct sweep (the rule and its
+// figures stand at use_direct in kernels.cu).
+bool direct_form(const sbiem_s* s, int shape) { return shape == 3 && (!s->fp32() || s->N > kFusedMaxN); }
+
+// Whether the direct sweep takes its weights from the table (FP32, on-chip
+// weights asked for and a table there).
+bool direct_gen(const sbiem_s* s, float gen_ds_max) {
+  return s->fp32() && gen_ds_max > 0.0f && s->direct_wtab != nullptr;
+}
+
+// Resident CTAs per SM of a sweep shape in the weight form of gen_ds_max.
+int sweep_blocks(const sbiem_s* s, int shape, float gen_ds_max) {
+  const bool gen = s->fp32() && s->f32.wtab && gen_ds_max > 0.0f;
+  int n;
+  if (direct_form(s, shape)) {
+    n = s->fp32() ? direct_blocks_per_sm<float>(direct_gen(s, gen_ds_max), s->direct_pieces, false)
+                  : direct_blocks_per_sm<double>(false, 0, false);
+  } else {
+    n = s->fp32() ? sweep_blocks_per_sm<float>(shape, gen) : sweep_blocks_per_sm<double>(shape, false);
+  }
+  return n < 1 ? 1 : n;
+}
+
+// Lags per item of the direct sweep: 2048, or as few as 256 while the handle
+// would have fewer than six items per resident warp (`warps`), so that the
+// last round of items stays a small part of the sweep.  A whole batch of rows
+// is 256 (FP32) or 128 (FP64) lags.
+int64_t direct_item_slots(const std::vector<int64_t>& Rn, int64_t warps) {
+  for (int64_t len = 2048; len > 256; len /= 2) {
+    int64_t n = 0;
+    for (int64_t r : Rn) n += (r + len - 1) / len;
+    if (n >= 6 * warps) return len;
+  }
+  return 256;
+}
+
+// Items of one fault's modes [in mode order], for `member` of an ensemble (0
+// for a single fault); w, w_off: the weights they read.
+template <class R>
+void direct_items_of(const sbiem_s* s, const DevFault<R>& f, const std::vector<int64_t>& w_off, int member, int64_t len,
+                     std::vector<DirectItem<R>>& items, std::vector<DirectRun>& runs) {
+  for (int n = 0; n < s->nmodes; ++n) {
+    const int64_t Rn = s->Rn[n], cnt = (Rn + len - 1) / len;
+    if (cnt > 1)
+      runs.push_back(DirectRun{static_cast<int32_t>(items.size()), static_cast<int32_t>(cnt), n, member});
+    const double ds = s->p.cs * (2.0 * M_PI * n / s->L) * s->dt_min / kDirectH;
+    DirectItem<R> it{};
+    it.ring = f.ring + s->ring_off[n];
+    it.w = f.w + w_off[n];
+    it.head = f.head + n;
+    it.Rn = static_cast<int32_t>(Rn);
+    it.mode = n;
+    it.member = member;
+    it.count = static_cast<int32_t>(cnt);
+    it.mt = static_cast<int32_t>(s->MT[n]);
+    it.mn = static_cast<int32_t>(s->MN[n]);
+    it.dh = static_cast<float>(ds);
+    it.dl = static_cast<float>(ds - static_cast<double>(it.dh));
+    for (int64_t c = 0; c < cnt; ++c) {
+      it.i0 = static_cast<int32_t>(c * len);
+      it.i1 = static_cast<int32_t>(std::min((c + 1) * len, Rn));
+      items.push_back(it);
+    }
+  }
+}
+
+// The handle's direct sweep: item and run tables on the device, partial sums
+// sized for them (f.partial also serves the bulk-async shapes' chunks).
+template <class R>
+int direct_setup(sbiem_s* s, DevFault<R>& f) {
+  std::vector<DirectItem<R>> items;
+  std::vector<DirectRun> runs;
+  direct_items_of<R>(s, f, s->w_off, 0, direct_item_slots(s->Rn, static_cast<int64_t>(s->sm_count) * 16), items, runs);
+  bool ok = true;
+  auto* d_items = alloc_n<DirectItem<R>>(s, std::max<size_t>(items.size(), 1), &ok);
+  auto* d_runs = alloc_n<DirectRun>(s, std::max<size_t>(runs.size(), 1), &ok);
+  if (items.size() > s->chunks.size()) f.partial = alloc_n<double4>(s, items.size(), &ok);
+  if (!ok) return nomem(s, "history sweep tables");
+  if (!items.empty())
+    CK(cudaMemcpyAsync(d_items, items.data(), sizeof(DirectItem<R>) * items.size(), cudaMemcpyHostToDevice, s->stream));
+  if (!runs.empty())
+    CK(cudaMemcpyAsync(d_runs, runs.data(), sizeof(DirectRun) * runs.size(), cudaMemcpyHostToDevice, s->stream));
+  CK(cudaStreamSynchronize(s->stream));  // the host vectors end here
+  f.direct.items = d_items;
+  f.direct.nitems = static_cast<int>(items.size());
+  f.direct.runs = d_runs;
+  f.direct.nruns = static_cast<int>(runs.size());
+  return SBIEM_OK;
+}
+
 // Grids and shapes of the two sweeps from sweep_shape, the weight form and
 // the CTAs per SM asked for.  Beside the one-launch FP32 pass the overlapped
-// sweep leaves each SM room for the pass kernels: with 2048-lag chunks
-// (shapes 3 and 4) shape 4 (one stage) on two CTAs per SM (with two stages
-// only one fits beside a pass CTA; flushed N = 4096 steps: 48-50 us with
-// one CTA per SM of the on-chip weight form, 41 us with two of the streamed
-// form); other shapes
-// one CTA per SM; with the four-kernel FFT (small CTAs) the full grid.
+// bulk-async sweep leaves each SM room for the pass kernels: with 2048-lag
+// chunks (shapes 3 and 4) shape 4 (one stage) on two CTAs per SM (with two
+// stages only one fits beside a pass CTA; flushed N = 4096 steps: 48-50 us
+// with one CTA per SM of the on-chip weight form, 41 us with two of the
+// streamed form); other shapes one CTA per SM; with the four-kernel FFT
+// the full grid.
 void sweep_config(sbiem_s* s) {
   const bool gen = s->fp32() && s->f32.wtab && s->gen_ds_max > 0.0f;
   s->f32.gen_ds_max = gen ? s->gen_ds_max : 0.0f;
-  int per_sm = s->fp32() ? sweep_blocks_per_sm<float>(s->sweep_shape, gen)
-                         : sweep_blocks_per_sm<double>(s->sweep_shape, false);
-  if (per_sm < 1) per_sm = 1;
+  const bool dgen = direct_gen(s, s->gen_ds_max);
+  s->f32.direct.wtab = dgen ? s->direct_wtab : nullptr;
+  s->f32.direct.pieces = dgen ? s->direct_pieces : 0;
+  int per_sm = sweep_blocks(s, s->sweep_shape, s->gen_ds_max);
   if (s->sweep_ctas > 0 && s->sweep_ctas < per_sm) per_sm = s->sweep_ctas;
   s->hist_grid = s->sm_count * per_sm;
   s->lag_shape = s->sweep_shape;
@@ -272,8 +368,7 @@ void sweep_config(sbiem_s* s) {
   }
   if (s->lag_ctas > 0) {
     // set by the autotuner: as many CTAs per SM as timed fastest beside the passes
-    const int lim = s->fp32() ? sweep_blocks_per_sm<float>(s->lag_shape, gen)
-                              : sweep_blocks_per_sm<double>(s->lag_shape, false);
+    const int lim = sweep_blocks(s, s->lag_shape, s->gen_ds_max);
     s->lag_grid = s->sm_count * std::max(1, std::min(s->lag_ctas, lim));
   }
   s->f64.sweep_shape = s->f32.sweep_shape = s->sweep_shape;
@@ -818,8 +913,20 @@ int sbiem_create(sbiem_t* out, const sbiem_params* pin, const double* h, const d
         s->gen_pieces = gp;
         s->gen_err = gerr;
         s->gen_ds_max = kGenDsMaxDefault;
+        // the direct sweep's table (lags below 2^23 keep (j + 1/2) exact in FP32)
+        if (*std::max_element(s->M.begin(), s->M.end()) < (int64_t(1) << 23)) {
+          std::vector<float> dtab;
+          build_direct_table(tab, s->dt_min, smax, dtab, &s->direct_pieces, &s->direct_err);
+          float4* d_dtab = alloc_n<float4>(s, dtab.size() / 4, &ok);
+          if (!ok || up(d_dtab, dtab.data(), sizeof(float) * dtab.size()) != cudaSuccess ||
+              cudaStreamSynchronize(s->stream) != cudaSuccess)
+            rc = nomem(s, "weight table");
+          else
+            s->direct_wtab = d_dtab;
+        }
       }
     }
+    if (rc == SBIEM_OK && direct_form(s, 3)) rc = direct_setup<float>(s, s->f32);
     sweep_config(s);
   } else {
     f.ring = alloc_n<Slot64>(s, static_cast<size_t>(std::max<int64_t>(s->total_slots, 1)), &ok);
@@ -833,7 +940,9 @@ int sbiem_create(sbiem_t* out, const sbiem_params* pin, const double* h, const d
     if (rc == SBIEM_OK) {
       launch_weights<double>(f, d_cheb, tab.npieces, tab.deg, tab.h, p.cs, d_MT, d_MN, p.quadrature, s->stream);
       launch_weight_pow2<double>(f, s->stream);
+      rc = direct_setup<double>(s, f);
     }
+    sweep_config(s);
   }
   if (rc == SBIEM_OK) rc = recompute_spectral_sums(s);
   if (rc == SBIEM_OK && cudaStreamSynchronize(s->stream) != cudaSuccess)
@@ -1539,9 +1648,13 @@ int sbiem_footprint(sbiem_t s, int64_t* hist_bytes, int64_t* device_bytes) {
   const int64_t slot = s->fp32() ? 16 : 32, wb = s->fp32() ? 8 : 16;
   // weights stream only for the modes that do not evaluate them on chip
   int64_t streamed = 0;
-  for (int n = 1; n < s->nmodes; ++n) {
+  // the direct sweep's table serves every mode, or none
+  const bool direct = s->fp32() && direct_form(s, s->sweep_shape);
+  const bool none = direct && s->f32.direct.wtab;
+  for (int n = 1; n < s->nmodes && !none; ++n) {
     const double ds = s->p.cs * (2.0 * M_PI * n / s->L) * s->dt_min;
-    if (!(s->fp32() && s->f32.gen_ds_max > 0.0f && static_cast<float>(ds) <= s->f32.gen_ds_max))
+    if (direct ||
+        !(s->fp32() && s->f32.gen_ds_max > 0.0f && static_cast<float>(ds) <= s->f32.gen_ds_max))
       streamed += s->Rn[n];
   }
   if (hist_bytes) *hist_bytes = s->total_slots * slot + streamed * wb;
@@ -1567,7 +1680,8 @@ int sbiem_get_sweep(sbiem_t s, int32_t* shape, double* gen_ds_max, int32_t* ctas
   if (gen_ds_max) *gen_ds_max = s->fp32() ? s->f32.gen_ds_max : 0.0;
   if (ctas_per_sm) *ctas_per_sm = s->hist_grid / (s->sm_count > 0 ? s->sm_count : 1);
   if (lag_ctas_per_sm) *lag_ctas_per_sm = s->lag_grid / (s->sm_count > 0 ? s->sm_count : 1);
-  if (table_err) *table_err = s->gen_pieces > 0 ? s->gen_err : -1.0;
+  if (table_err)
+    *table_err = s->gen_pieces <= 0 ? -1.0 : (direct_form(s, s->sweep_shape) && s->direct_wtab ? s->direct_err : s->gen_err);
   return SBIEM_OK;
 }
 
@@ -1625,8 +1739,9 @@ int sbiem_tune(sbiem_t s, int reps, int32_t* shape_out, double* gen_out, int32_t
   for (int shape = 0; shape <= 4; ++shape) {
     if (sweep_chunk_slots(s->p.precision, shape) != s->chunk_slots) continue;
     for (float t : thr) {
-      const int lim = s->fp32() ? sweep_blocks_per_sm<float>(shape, t > 0.0f)
-                                : sweep_blocks_per_sm<double>(shape, false);
+      // the direct sweep's table serves every mode: one threshold stands for all
+      if (direct_form(s, shape) && t > 0.0f && t != kGenDsMaxDefault) continue;
+      const int lim = sweep_blocks(s, shape, t);
       for (int c = 1; c <= lim; ++c) {
         s->sweep_shape = shape;
         s->gen_ds_max = t;
@@ -1753,8 +1868,7 @@ int sbiem_tune(sbiem_t s, int reps, int32_t* shape_out, double* gen_out, int32_t
     CK(cudaStreamSynchronize(s->stream));
     s->lag_ctas = 0;
     sweep_config(s);
-    const int lim = s->fp32() ? sweep_blocks_per_sm<float>(s->lag_shape, s->f32.gen_ds_max > 0.0f)
-                              : sweep_blocks_per_sm<double>(s->lag_shape, false);
+    const int lim = sweep_blocks(s, s->lag_shape, s->gen_ds_max);
     float lbest = 1e30f;
     int lb = 0;
     // nine timed launches at least: the candidates' totals are close (with
@@ -1850,6 +1964,12 @@ struct sbiem_batch_s {
     int n;
   };
   std::map<int64_t, ChunkSet> sets;
+  // the direct sweep (shape 3): the members' items laid end to end
+  DirectTable<double> direct64{};
+  DirectTable<float> direct32{};
+  double4* direct_partial = nullptr;
+  const float4* direct_wtab = nullptr;  // the widest member's table (NULL: streamed)
+  int direct_pieces = 0;
   int2* mm = nullptr;           // (member, mode) pairs of the per-mode sums
   int TM = 0;
   int shape = 0;                // sweep shape shared by the members
@@ -1980,6 +2100,54 @@ int batch_use_chunks(sbiem_batch_s* b, int64_t slots) {
   return SBIEM_OK;
 }
 
+// Whether the ensemble's direct sweep takes its weights from the table.
+bool batch_direct_gen(const sbiem_batch_s* b) { return b->fp32 && b->gen && b->direct_wtab; }
+
+// Resident CTAs per SM of the ensemble's history launch in a sweep shape.
+int batch_blocks(const sbiem_batch_s* b, int shape, bool gen) {
+  int n;
+  if (shape == 3)
+    n = b->fp32 ? direct_blocks_per_sm<float>(gen && b->direct_wtab, b->direct_pieces, true)
+                : direct_blocks_per_sm<double>(false, 0, true);
+  else
+    n = b->fp32 ? persist_blocks_per_sm<float>(shape, gen) : persist_blocks_per_sm<double>(shape, false);
+  return n < 1 ? 1 : n;
+}
+
+template <class R>
+DirectTable<R>& batch_direct(sbiem_batch_s* b) {
+  if constexpr (sizeof(R) == 8) return b->direct64;
+  else return b->direct32;
+}
+
+// Items of every member (fs: their descriptors, with the weights each reads),
+// and the partial sums.
+template <class R>
+int batch_direct_setup(sbiem_batch_s* b, const std::vector<DevFault<R>>& fs,
+                       const std::vector<std::vector<int64_t>>& w_off) {
+  std::vector<int64_t> all;
+  for (const auto* m : b->members) all.insert(all.end(), m->Rn.begin(), m->Rn.end());
+  const int64_t len = direct_item_slots(all, static_cast<int64_t>(b->sm_count) * 16);
+  std::vector<DirectItem<R>> items;
+  std::vector<DirectRun> runs;
+  for (size_t r = 0; r < b->members.size(); ++r)
+    direct_items_of<R>(b->members[r], fs[r], w_off[r], static_cast<int>(r), len, items, runs);
+  if (items.size() > static_cast<size_t>(1) << 30) return fail(SBIEM_ERR_INVALID, "batch: too many history items");
+  auto* d_items = static_cast<DirectItem<R>*>(batch_alloc(b, sizeof(DirectItem<R>) * std::max<size_t>(items.size(), 1)));
+  auto* d_runs = static_cast<DirectRun*>(batch_alloc(b, sizeof(DirectRun) * std::max<size_t>(runs.size(), 1)));
+  b->direct_partial = static_cast<double4*>(batch_alloc(b, sizeof(double4) * std::max<size_t>(items.size(), 1)));
+  if (!d_items || !d_runs || !b->direct_partial)
+    return fail(SBIEM_ERR_NOMEM, "batch: device allocation failed (history items)");
+  if (!items.empty()) CK(cudaMemcpy(d_items, items.data(), sizeof(DirectItem<R>) * items.size(), cudaMemcpyHostToDevice));
+  if (!runs.empty()) CK(cudaMemcpy(d_runs, runs.data(), sizeof(DirectRun) * runs.size(), cudaMemcpyHostToDevice));
+  auto& t = batch_direct<R>(b);
+  t.items = d_items;
+  t.nitems = static_cast<int>(items.size());
+  t.runs = d_runs;
+  t.nruns = static_cast<int>(runs.size());
+  return SBIEM_OK;
+}
+
 template <class R>
 int batch_build(sbiem_batch_s* b) {
   std::vector<int2> mm;
@@ -2003,6 +2171,8 @@ int batch_build(sbiem_batch_s* b) {
   }
   // weights: each member reads those of the largest member it can (itself
   // when none); members of one size share one offset table into it
+  std::vector<std::vector<int64_t>> w_off(b->members.size());
+  for (size_t r = 0; r < b->members.size(); ++r) w_off[r] = b->members[r]->w_off;
   {
     const size_t nm = b->members.size();
     std::map<std::pair<size_t, int64_t>, int64_t*> maps;  // (source member, N) -> device offsets
@@ -2024,13 +2194,13 @@ int batch_build(sbiem_batch_s* b) {
         fs[r].wgen = fs[src].wgen;
         continue;
       }
+      for (int n = 0; n <= sr->nmodes; ++n)
+        w_off[r][n] = b->members[src]->w_off[std::min<size_t>(static_cast<size_t>(n) * ratio,
+                                                              static_cast<size_t>(b->members[src]->nmodes))];
       auto key = std::make_pair(src, static_cast<int64_t>(sr->p.N));
       auto it = maps.find(key);
       if (it == maps.end()) {
-        const sbiem_s* sc = b->members[src];
-        std::vector<int64_t> wo(static_cast<size_t>(sr->nmodes) + 1);
-        for (int n = 0; n <= sr->nmodes; ++n)
-          wo[n] = sc->w_off[std::min<size_t>(static_cast<size_t>(n) * ratio, static_cast<size_t>(sc->nmodes))];
+        const std::vector<int64_t>& wo = w_off[r];
         int64_t* d = static_cast<int64_t*>(batch_alloc(b, sizeof(int64_t) * wo.size()));
         if (!d) return fail(SBIEM_ERR_NOMEM, "batch: device allocation failed (weight offsets)");
         CK(cudaMemcpy(d, wo.data(), sizeof(int64_t) * wo.size(), cudaMemcpyHostToDevice));
@@ -2051,7 +2221,7 @@ int batch_build(sbiem_batch_s* b) {
   CK(cudaMemcpyAsync(b->fs, fs.data(), sizeof(DevFault<R>) * fs.size(), cudaMemcpyHostToDevice, b->stream));
   CK(cudaStreamSynchronize(b->stream));
   b->TM = static_cast<int>(mm.size());
-  return SBIEM_OK;
+  return batch_direct_setup<R>(b, fs, w_off);
 }
 
 // Whole-window sums of every member (AT, AN), or with ahead = true the next
@@ -2062,8 +2232,17 @@ void batch_history(sbiem_batch_s* b, cudaStream_t st, bool ahead = false) {
   // occupancy the CTAs per SM were chosen within) and at least one chunk each
   int grid = ahead ? b->lag_grid : b->hist_grid;
   const bool gen = sizeof(R) == 4 && b->gen;
-  const int resident = b->sm_count * std::max(1, persist_blocks_per_sm<R>(b->shape, gen));
+  const int resident = b->sm_count * batch_blocks(b, b->shape, gen);
   if (grid > resident) grid = resident;
+  if (b->shape == 3) {
+    auto t = batch_direct<R>(b);
+    t.wtab = batch_direct_gen(b) ? b->direct_wtab : nullptr;
+    t.pieces = t.wtab ? b->direct_pieces : 0;
+    const SweepBarrier bar{b->bar, b->bar + 1, b->bar_limit, static_cast<int>(b->members.size())};
+    launch_direct_batch<R>(t, static_cast<const DevFault<R>*>(b->fs), b->direct_partial, ahead ? 2 : 1, grid, ahead,
+                           b->persistent, bar, st);
+    return;
+  }
   if (grid > b->nchunks) grid = b->nchunks > 0 ? b->nchunks : 1;
   if (!b->persistent) {
     launch_history_batch<R>(static_cast<const DevFault<R>*>(b->fs), b->chunks, b->nchunks, b->partial, b->mm,
@@ -2176,19 +2355,21 @@ int sbiem_batch_create(sbiem_batch_t* out, int n, const sbiem_t* members, int64_
     const sbiem_s* widest = members[0];
     for (int r = 0; r < n; ++r) {
       const sbiem_s* m = members[r];
-      same = same && m->f32.wtab && m->p.cs / m->p.cp == members[0]->p.cs / members[0]->p.cp &&
+      same = same && m->f32.wtab && (m->direct_wtab != nullptr) == (members[0]->direct_wtab != nullptr) && m->p.cs / m->p.cp == members[0]->p.cs / members[0]->p.cp &&
              m->dt_min == members[0]->dt_min;
       if (m->gen_pieces > widest->gen_pieces) widest = m;
     }
     if (same) {
       b->wtab = widest->f32.wtab;
       b->gen_pieces = widest->gen_pieces;
+      b->direct_wtab = widest->direct_wtab;
+      b->direct_pieces = widest->direct_pieces;
       b->gen = true;
       b->gen_ds_max = kGenDsMaxDefault;
     }
   }
-  b->per_sm_plain = fp32 ? persist_blocks_per_sm<float>(b->shape, false) : persist_blocks_per_sm<double>(b->shape, false);
-  b->per_sm_gen = b->gen ? persist_blocks_per_sm<float>(b->shape, true) : 0;
+  b->per_sm_plain = batch_blocks(b, b->shape, false);
+  b->per_sm_gen = b->gen ? batch_blocks(b, b->shape, true) : 0;
   if (b->per_sm_plain < 1) b->per_sm_plain = 1;
   if (b->per_sm_gen < 1) b->per_sm_gen = 1;
   b->per_sm = b->gen ? b->per_sm_gen : b->per_sm_plain;
@@ -2210,7 +2391,7 @@ int sbiem_batch_create(sbiem_batch_t* out, int n, const sbiem_t* members, int64_
     // the overlapped sweep leaves room for the one-launch FP32 passes
     bool small = fp32;
     for (auto* m : b->members) small = small && m->N <= kFusedMaxN;
-    b->lag_grid = small ? b->sm_count : b->hist_grid;
+    b->lag_grid = small && b->shape != 3 ? b->sm_count : b->hist_grid;
   }
   for (auto* m : b->members) cudaStreamSynchronize(m->stream);
   int rc = fp32 ? batch_build<float>(b) : batch_build<double>(b);
@@ -2365,9 +2546,8 @@ int sbiem_batch_tune(sbiem_batch_t b, int reps, int64_t* chunk_out, int* blocks_
     b->shape = sh;
     b->gen = tv > 0.0f;
     b->gen_ds_max = tv;
-    const int lim = b->gen ? persist_blocks_per_sm<float>(sh, true)
-                           : (b->fp32 ? persist_blocks_per_sm<float>(sh, false)
-                                      : persist_blocks_per_sm<double>(sh, false));
+    if (sh == 3 && tv > 0.0f && tv != kGenDsMaxDefault) continue;  // one threshold stands for all
+    const int lim = batch_blocks(b, sh, b->gen);
     for (int bl = 1; bl <= lim; ++bl) {
       b->hist_grid = b->sm_count * bl;
       // one untimed launch, then reps timed ones; take the median
@@ -2402,9 +2582,8 @@ int sbiem_batch_tune(sbiem_batch_t b, int reps, int64_t* chunk_out, int* blocks_
   }
   b->gen = best_gen;
   b->gen_ds_max = best_thr;
-  b->per_sm_plain = b->fp32 ? persist_blocks_per_sm<float>(b->shape, false)
-                            : persist_blocks_per_sm<double>(b->shape, false);
-  b->per_sm_gen = b->gen ? persist_blocks_per_sm<float>(b->shape, true) : b->per_sm_gen;
+  b->per_sm_plain = batch_blocks(b, b->shape, false);
+  b->per_sm_gen = b->gen ? batch_blocks(b, b->shape, true) : b->per_sm_gen;
   b->per_sm = b->gen ? b->per_sm_gen : b->per_sm_plain;
   b->hist_grid = b->sm_count * best_b;
   // The history form (one persistent launch or two launches; they agree
@@ -2446,9 +2625,7 @@ int sbiem_batch_tune(sbiem_batch_t b, int reps, int64_t* chunk_out, int* blocks_
       else batch_passes<double>(b, b->stream, b->ev_fork);
     }, &t_pass);
     if (rc) return rc;
-    const int lim = b->gen ? persist_blocks_per_sm<float>(b->shape, true)
-                           : (b->fp32 ? persist_blocks_per_sm<float>(b->shape, false)
-                                      : persist_blocks_per_sm<double>(b->shape, false));
+    const int lim = batch_blocks(b, b->shape, b->gen);
     float t_best = 1e30f, t_sweep_kept = best;
     bool ov_best = false, pers_best = true;
     int lag_best = b->lag_grid;

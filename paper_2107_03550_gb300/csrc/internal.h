@@ -28,9 +28,16 @@ constexpr double kGenDsBlockMax = kGenH / 16.0;
 // kGenDsBlockMax and up to this).
 constexpr double kGenDsBlock4Max = kGenH / 8.0;
 
+// Weight table of the direct sweep (per lag, so no span beyond the piece):
+// piece width and degree.
+constexpr double kDirectH = 0.125;
+constexpr int kDirectDeg = 4;
+
 void kernel_values(double s, double r, double* cT, double* cN);
 void build_gen_table(double r, double dt, double smax, std::vector<float>& tab, int* npieces, double* max_err);
 void build_cheb(double r, double smax, ChebTable* tab);
+void build_direct_table(const ChebTable& cheb, double dt, double smax, std::vector<float>& tab, int* npieces,
+                        double* max_err);
 void build_twiddles(int64_t N, std::vector<double>& tw);
 
 }  // namespace sbiem

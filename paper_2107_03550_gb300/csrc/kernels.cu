@@ -15,6 +15,7 @@
 #include <cstdint>
 #include <type_traits>
 
+#include "device.cuh"
 #include "internal.h"
 #include "kernels.cuh"
 #include <math_constants.h>
@@ -31,19 +32,6 @@ template <class C> __device__ __forceinline__ C cmul(C a, C b) {
   r.x = a.x * b.x - a.y * b.y;
   r.y = a.x * b.y + a.y * b.x;
   return r;
-}
-
-// Programmatic dependent launch: a kernel launched with the programmatic
-// serialization attribute may start while its predecessor runs; it must
-// read nothing the predecessor chain writes before pdl_wait() returns.
-// pdl_trigger() lets this kernel's own dependent start launching.  Both are
-// no-ops for a kernel launched without the attribute.
-__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-
-// Shared-memory address of a generic pointer into this CTA's shared memory.
-__device__ __forceinline__ uint32_t smem_u32(const void* p) {
-  return static_cast<uint32_t>(__cvta_generic_to_shared(p));
 }
 
 // --------------------------------------------------------- shared-memory FFT
@@ -953,6 +941,8 @@ __global__ void __launch_bounds__(kHistThreads)
 // shape 1: twice the lags; shape 2: twice the stages; shape 3: 4x the lags, 2
 // stages; shape 4: shape 3's chunks in one stage (49 KB), for the sweep that
 // runs beside the spectral passes: two of its CTAs and a pass CTA share an SM.
+// Where the direct sweep (direct.cu) is the better form it takes shape 3's
+// place (use_direct).
 template <class R, int SH> struct SweepCfg {
   static constexpr int kBase = sizeof(R) == 4 ? 512 : 256;
   static constexpr int kSlots = SH == 1 ? 2 * kBase : (SH >= 3 ? 4 * kBase : kBase);
@@ -981,19 +971,6 @@ constexpr int kGenF4 = kGenPairs / 2;
 static_assert(kGenPairs % 2 == 0, "coefficient pairs come two per float4");
 constexpr float kGenHf = static_cast<float>(kGenH);
 constexpr float kGenInvH = static_cast<float>(1.0 / kGenH);
-
-// Two FP32 fused multiply-adds in one packed instruction (fma.rn.f32x2):
-// each lane rounds exactly as fmaf does.
-__device__ __forceinline__ float2 ffma2(float2 a, float2 b, float2 c) {
-  unsigned long long ra, rb, rc, rd;
-  asm("mov.b64 %0, {%1, %2};" : "=l"(ra) : "f"(a.x), "f"(a.y));
-  asm("mov.b64 %0, {%1, %2};" : "=l"(rb) : "f"(b.x), "f"(b.y));
-  asm("mov.b64 %0, {%1, %2};" : "=l"(rc) : "f"(c.x), "f"(c.y));
-  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(rd) : "l"(ra), "l"(rb), "l"(rc));
-  float2 d;
-  asm("mov.b64 {%0, %1}, %2;" : "=f"(d.x), "=f"(d.y) : "l"(rd));
-  return d;
-}
 
 // The weights of a thread's block of kGenBlock consecutive lags come from
 // one piece: the block starts at lag j (s0 = (j + 1/2) ds, ds = dsh + dsl as
@@ -1082,16 +1059,6 @@ __device__ __forceinline__ uint64_t l2_policy_evict_first() {
   asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(pol));
   return pol;
 }
-
-// s + c += a with the rounding error of the addition carried in c (Knuth's
-// TwoSum; FP32 only -- an FP64 sum needs no compensation here).
-__device__ __forceinline__ void two_sum_add(float& s, float& c, float a) {
-  const float t = s + a;
-  const float bb = t - s;
-  c += (s - (t - bb)) + (a - bb);
-  s = t;
-}
-__device__ __forceinline__ void two_sum_add(double& s, double& /*c*/, double a) { s += a; }
 
 // Fixed-order tree sum of a warp's values, valid in lane 0.  Only the lanes
 // that keep a partial sum add (lane < o), so the FP64 pipe (scarce on GB300)
@@ -1501,25 +1468,15 @@ __global__ void k_sweep_finish_b(const DevFault<R>* __restrict__ fs, const int2*
 // SBIEM_FLAG_WAIT on every member and leaves (their steps are rejected,
 // nothing is committed); a CTA whose copy wait gave up flags the members of
 // the chunks it did not sum and still arrives.
-struct SweepBarrier {
-  unsigned* count;
-  unsigned* epoch;
-  long long limit;
-  int members;
-};
-
 template <class R, int SH, bool GEN>
 __global__ void __launch_bounds__(sweep_threads(GEN), GEN ? 4 : 1)
     k_sweep_persist(const DevFault<R>* __restrict__ fs, const Chunk* __restrict__ chunks, int nch,
                     double4* __restrict__ partial, int m_dt, const float4* __restrict__ wtab, int wtab_pieces,
                     float gen_ds_max, const int2* __restrict__ mm, int TM, const int2* __restrict__ fc,
                     bool ahead, const SweepBarrier bar, bool ring_evict_first) {
-  __shared__ unsigned s_epoch, s_fail;
+  __shared__ unsigned s_epoch;
   const int tid = threadIdx.x;
-  if (tid == 0) {
-    s_epoch = *reinterpret_cast<volatile unsigned*>(bar.epoch);
-    s_fail = 0u;
-  }
+  if (tid == 0) s_epoch = *reinterpret_cast<volatile unsigned*>(bar.epoch);
   __syncthreads();
   const int c0 = static_cast<int>(static_cast<int64_t>(blockIdx.x) * nch / gridDim.x);
   const int c1 = static_cast<int>(static_cast<int64_t>(blockIdx.x + 1) * nch / gridDim.x);
@@ -1531,33 +1488,7 @@ __global__ void __launch_bounds__(sweep_threads(GEN), GEN ? 4 : 1)
     if (!ok && tid == 0)
       for (int c = c0 + k_stop; c < c1; ++c) atomicOr(fs[chunks[c].pad].status, SBIEM_FLAG_WAIT);
   }
-  // grid barrier (bounded)
-  __syncthreads();
-  if (tid == 0) {
-    __threadfence();  // this CTA's partials before its arrival
-    const unsigned ticket = atomicAdd(bar.count, 1u);
-    if (ticket == gridDim.x - 1) {
-      *reinterpret_cast<volatile unsigned*>(bar.count) = 0u;
-      __threadfence();
-      atomicAdd(bar.epoch, 1u);
-    } else {
-      bool released = false;
-      for (long long q = 0; q < bar.limit; ++q) {
-        if (*reinterpret_cast<volatile unsigned*>(bar.epoch) != s_epoch) {
-          released = true;
-          break;
-        }
-        __nanosleep(64);
-      }
-      if (!released) {
-        s_fail = 1u;
-        for (int r = 0; r < bar.members; ++r) atomicOr(fs[r].status, SBIEM_FLAG_WAIT);
-      }
-    }
-    __threadfence();
-  }
-  __syncthreads();
-  if (s_fail) return;
+  if (!grid_barrier<R>(fs, bar, s_epoch)) return;
   for (int t = blockIdx.x * blockDim.x + tid; t < TM; t += gridDim.x * blockDim.x)
     finish_pair<R>(fs, mm, t, fc, nch, gridDim.x, partial, ahead);
 }
@@ -2510,8 +2441,22 @@ static void launch_finish(const DevFault<R>& f, double2* outT, double2* outN, bo
   launch_early(k_sweep_finish<R>, dim3((f.nmodes + 255) / 256), dim3(256), 0, st, fv, outT, outN, f32, G);
 }
 
+// Shape 3 is the direct sweep in FP64 and, in FP32, above kFusedMaxN (sweep
+// alone, direct against bulk-async: FP64 N = 1024 12.5 and 24.9 us, 8192 68
+// and 129 us, 65536 513 and 1210 us; FP32 N = 65536 183 and 222 us, 262144 782
+// and 980 us; at N = 4096 21.0 and 18.5 us).  A caller's own copy-wait limit
+// asks for the form that has such waits.
+template <class R>
+static bool use_direct(const DevFault<R>& f, int shape) {
+  return shape == 3 && (sizeof(R) == 8 || f.N > kFusedMaxN) && f.spin_limit == kSpinLimit;
+}
+
 template <class R>
 void launch_history(const DevFault<R>& f, int m_dt, int grid, cudaStream_t st, cudaEvent_t sweep_done) {
+  if (use_direct(f, f.sweep_shape)) {
+    launch_direct<R>(f.direct, f, m_dt, grid, false, st, sweep_done);
+    return;
+  }
   launch_sweep<R>(f, m_dt, grid, f.sweep_shape, st);
   if (sweep_done) cudaEventRecord(sweep_done, st);
   launch_finish<R>(f, f.AT, f.AN, true, grid, st);
@@ -2520,6 +2465,10 @@ void launch_history(const DevFault<R>& f, int m_dt, int grid, cudaStream_t st, c
 template <class R>
 void launch_history_ahead(const DevFault<R>& f, int m_dt, int grid, cudaStream_t st) {
   // into BT/BN; the commit adds the new slot's term
+  if (use_direct(f, f.lag_shape)) {
+    launch_direct<R>(f.direct, f, 2 * m_dt, grid, true, st, nullptr);
+    return;
+  }
   launch_sweep<R>(f, 2 * m_dt, grid, f.lag_shape, st);
   launch_finish<R>(f, f.BT, f.BN, false, grid, st);
 }
@@ -2820,6 +2769,7 @@ void launch_real_part(int N, const double2* z, double* x, cudaStream_t st) {
 
 template <class R>
 void configure_kernels(const FftGeom& g) {
+  configure_direct<R>();
   for (int sh = 0; sh < kSweepShapes; ++sh)
     with_shape(sh, [&](auto shc) {
       constexpr int SH = decltype(shc)::value;

@@ -2,6 +2,7 @@
 #pragma once
 #include <cuda_runtime.h>
 #include <cstdint>
+#include <type_traits>
 
 #include "mlp.cuh"
 #include "sbiem.h"
@@ -43,6 +44,33 @@ struct Chunk {
 // (length N1); B columns or rows per CTA.
 struct FftGeom {
   int N, N1, N2, lgN1, lgN2, Bc, Br, tc, tr;
+};
+
+// ---------------------------------------- direct sweep (direct.cu): its tables
+// One item: consecutive history slots [i0, i1) of one mode, with everything
+// static that the sweep needs of it (one 64-byte record).
+template <class R>
+struct __align__(64) DirectItem {
+  const void* ring;    // the mode's ring
+  const W2<R>* w;      // its weights
+  const int32_t* head; // where its ring head is kept
+  int32_t i0, i1, Rn;
+  int32_t mode, member, count;  // count: items of this mode
+  int32_t mt, mn;      // the two fields' windows
+  float dh, dl;        // ds = c_s k_n dt_min over the piece width, as two floats
+};
+// A mode of several items: their sums are added up after the sweep.
+struct DirectRun {
+  int32_t first, count, mode, member;
+};
+template <class R>
+struct DirectTable {
+  const DirectItem<R>* items = nullptr;
+  int nitems = 0;
+  const DirectRun* runs = nullptr;
+  int nruns = 0;
+  const float4* wtab = nullptr;  // weight table (FP32; NULL: the weights are streamed)
+  int pieces = 0;
 };
 
 // Pointers of one fault on the device.
@@ -88,7 +116,7 @@ struct DevFault {
   const Chunk* chunks;
   int nchunks;
   const int32_t *mfirst, *mcount;          // per mode: first chunk, chunks
-  int sweep_shape;                         // chunk length x stages of the history sweep (0..3)
+  int sweep_shape;                         // form of the history sweep (0..4; 3: the direct sweep)
   int lag_shape;                           // the same for the sweep beside the passes (0..4)
   // FP32 sweep with the weights evaluated on chip instead of streamed:
   // per mode (ds_hi, ds_lo, M^T bits, M^N bits) with ds = c_s k_n dt_min as
@@ -115,7 +143,9 @@ struct DevFault {
   unsigned long long* harvest_count;
   long long harvest_cap;
   int* work;                               // next chunk of the history convolution
+  DirectTable<R> direct;                   // items and weight table of the direct sweep
 };
+
 
 // One-launch FP32 spectral pass: a single CTA of N/8 threads below
 // kClusterMinN, a cluster of cluster_ctas(N) CTAs from kClusterMinN to
@@ -139,6 +169,28 @@ __host__ __device__ constexpr int batch_cluster_ctas(int N) { return N >= 16384 
 #define SBIEM_CLUSTER_EPT 4
 #endif
 constexpr int kClusterEPT = SBIEM_CLUSTER_EPT;
+
+// Grid barrier of the ensemble's persistent launches: counter and epoch in
+// device memory, the polls of the epoch before a CTA gives up, and the
+// members to flag then.
+struct SweepBarrier {
+  unsigned* count;
+  unsigned* epoch;
+  long long limit;
+  int members;
+};
+template <class R> void configure_direct();
+// Resident CTAs per SM of the direct sweep (gen: with a weight table of
+// `pieces` pieces).
+template <class R> int direct_blocks_per_sm(bool gen, int pieces, bool persist);
+// History sums of a step of m dt_min into AT/AN (ahead: BT/BN, the caller
+// passes the doubled shift); `swept` (may be NULL) is recorded between the
+// sweep and the sums of the modes of several items.
+template <class R> void launch_direct(const DirectTable<R>& t, const DevFault<R>& f, int m, int grid, bool ahead,
+                                      cudaStream_t st, cudaEvent_t swept);
+template <class R> void launch_direct_batch(const DirectTable<R>& t, const DevFault<R>* fs, double4* partial, int m,
+                                            int grid, bool ahead, bool persistent, const SweepBarrier& bar,
+                                            cudaStream_t st);
 
 // Host launch wrappers (kernels.cu).
 // Plain streaming read of `bytes` (16-byte aligned; sbiem_read_probe).

@@ -22,6 +22,7 @@
 //   with s = c_s k t, r = c_s/c_p, A = (1/r^2 - 2)^2 r^2 / 2 (Eq. Ct and the
 //   C^N expression of Sec. 2.4 regrouped so that no two large terms cancel).
 //   J0, J1 are the C library's j0/j1.
+#include <algorithm>
 #include <cmath>
 #include <vector>
 
@@ -287,6 +288,84 @@ void build_gen_table(double r, double dt, double smax, std::vector<float>& tab, 
       kernel_values(a + half * (t + 1.0), r, &cT, &cN);
       err = std::max(err, std::max(std::fabs(eT - dt * cT), std::fabs(eN - dt * cN)));
       cmax = std::max(cmax, std::max(std::fabs(cT), std::fabs(cN)));
+    }
+  }
+  *max_err = cmax > 0.0 ? err / (dt * cmax) : 0.0;
+}
+
+namespace {
+// (C^T, C^N)(s) from the Chebyshev table (Clenshaw).
+void cheb_eval(const ChebTable& c, double s, double* cT, double* cN) {
+  const int p = std::min(static_cast<int>(s / c.h), c.npieces - 1);
+  const double t = 2.0 * (s - p * c.h) / c.h - 1.0;
+  const double* a = &c.coef[static_cast<size_t>(p) * (c.deg + 1) * 2];
+  double T1 = 0.0, T2 = 0.0, N1 = 0.0, N2 = 0.0;
+  for (int k = c.deg; k >= 1; --k) {
+    const double x = 2.0 * t * T1 - T2 + a[2 * k], y = 2.0 * t * N1 - N2 + a[2 * k + 1];
+    T2 = T1;
+    T1 = x;
+    N2 = N1;
+    N1 = y;
+  }
+  *cT = t * T1 - T2 + a[0];
+  *cN = t * N1 - N2 + a[1];
+}
+}  // namespace
+
+// FP32 table of the weights dt C(s) for the direct sweep.  Piece q is centred
+// at s = q kDirectH and serves |s - q kDirectH| <= kDirectH / 2 (piece 0: s >=
+// 0): a polynomial of degree kDirectDeg in u = s / kDirectH - q, |u| <= 1/2,
+// interpolating at the Chebyshev nodes of that range.  Layout for P pieces:
+// P x (c0T, c0N, c1T, c1N), P x (c2T, c2N, c3T, c3N), P x (c4T, c4N).
+// Interpolation error: |C^(5)| (kDirectH / 2)^5 / (5! 2^4), with the kernels
+// oscillating at up to 1/r in s about 5e-9 of max|C|.  *max_err: the largest
+// |table - dt C| over 16 points per piece, evaluated in FP64 from the rounded
+// coefficients, over dt max|C|.
+void build_direct_table(const ChebTable& cheb, double dt, double smax, std::vector<float>& tab, int* npieces,
+                        double* max_err) {
+  constexpr int n = kDirectDeg + 1;
+  static_assert(n == 5, "the layout below holds five coefficients");
+  const int P = static_cast<int>(std::ceil(smax / kDirectH)) + 2;
+  *npieces = P;
+  tab.assign((static_cast<size_t>(2) * P + (P + 1) / 2) * 4, 0.0f);
+  double err = 0.0, cmax = 0.0;
+  for (int q = 0; q < P; ++q) {
+    // nodes in u: the piece's half of the range where it starts at s = 0
+    const double lo = q == 0 ? 0.0 : -0.5, hi = 0.5;
+    double x[n], c[2][n];
+    for (int i = 0; i < n; ++i) {
+      x[i] = 0.5 * (lo + hi) + 0.5 * (hi - lo) * std::cos(M_PI * (i + 0.5) / n);
+      cheb_eval(cheb, (q + x[i]) * kDirectH, &c[0][i], &c[1][i]);
+    }
+    for (int f = 0; f < 2; ++f) {
+      // Newton's divided differences, then to powers of u
+      double d[n];
+      for (int i = 0; i < n; ++i) d[i] = c[f][i];
+      for (int k = 1; k < n; ++k)
+        for (int i = n - 1; i >= k; --i) d[i] = (d[i] - d[i - 1]) / (x[i] - x[i - k]);
+      double a[n] = {0.0};
+      for (int k = n - 1; k >= 0; --k) {
+        // a <- a (u - x_k) + d_k
+        for (int i = n - 1; i >= 1; --i) a[i] = a[i - 1] - x[k] * a[i];
+        a[0] = d[k] - x[k] * a[0];
+      }
+      for (int k = 0; k < 4; ++k)
+        tab[4 * (static_cast<size_t>(k / 2) * P + q) + 2 * (k & 1) + f] = static_cast<float>(dt * a[k]);
+      tab[static_cast<size_t>(8) * P + 2 * q + f] = static_cast<float>(dt * a[4]);
+    }
+    for (int i = 0; i < 16; ++i) {
+      const double u = lo + (hi - lo) * (i + 0.5) / 16.0;
+      double v[2];
+      cheb_eval(cheb, (q + u) * kDirectH, &v[0], &v[1]);
+      for (int f = 0; f < 2; ++f) {
+        const size_t P4 = static_cast<size_t>(4) * P;
+        const double a[n] = {tab[4 * q + f], tab[4 * q + 2 + f], tab[P4 + 4 * q + f], tab[P4 + 4 * q + 2 + f],
+                             tab[2 * P4 + 2 * q + f]};
+        double w = a[4];
+        for (int k = 3; k >= 0; --k) w = w * u + a[k];
+        err = std::max(err, std::fabs(w - dt * v[f]));
+        cmax = std::max(cmax, std::fabs(v[f]));
+      }
     }
   }
   *max_err = cmax > 0.0 ? err / (dt * cmax) : 0.0;
