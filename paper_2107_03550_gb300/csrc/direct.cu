@@ -107,21 +107,6 @@ __device__ __forceinline__ void direct_fma(Acc64& a, const Slot64& s, const doub
   a.n.y = fma(w.y, s.n.y, a.n.y);
 }
 
-// Sum of four values over the warp with 9 additions instead of 20 (the FP64
-// pipe is scarce): lanes exchange halves of the set first, so after two
-// rounds a lane carries one value.  Lane 8 q returns value q; fixed order.
-template <class T>
-__device__ __forceinline__ T warp_reduce4(T v0, T v1, T v2, T v3) {
-  const int lane = threadIdx.x & 31;
-  const bool up = lane & 16, odd = lane & 8;
-  const T a = (up ? v2 : v0) + __shfl_xor_sync(0xffffffffu, up ? v0 : v2, 16);
-  const T b = (up ? v3 : v1) + __shfl_xor_sync(0xffffffffu, up ? v1 : v3, 16);
-  T r = (odd ? b : a) + __shfl_xor_sync(0xffffffffu, odd ? a : b, 8);
-#pragma unroll
-  for (int o = 4; o > 0; o >>= 1) r += __shfl_xor_sync(0xffffffffu, r, o);
-  return r;
-}
-
 // (w^T, w^N) at lag jf - 1/2 from the table in shared memory (P pieces): dh
 // + dl is ds over the piece width.
 __device__ __forceinline__ float2 table_weight(const float4* __restrict__ tab, int P, float jf, float dh, float dl) {

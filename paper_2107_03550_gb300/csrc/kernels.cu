@@ -877,28 +877,28 @@ __global__ void __launch_bounds__(kHistThreads)
         if (i + 32 * u < iend) slot_fma(acc, sv[u], wv[u]);
     }
     // reduce in the accumulation precision (FP32 partial sums in the precision
-    // form), widen once per chunk for the cross-chunk sum
-    const double4 v = make_double4(static_cast<double>(warp_sum(acc.tr)), static_cast<double>(warp_sum(acc.ti)),
-                                   static_cast<double>(warp_sum(acc.nr)), static_cast<double>(warp_sum(acc.ni)));
+    // form); lane 8 q holds value q (shear re, im, normal re, im), widened
+    // once per chunk for the cross-chunk sum
+    const double v = static_cast<double>(warp_reduce4<R>(acc.tr, acc.ti, acc.nr, acc.ni));
+    const bool mine = (lane & 7) == 0;
+    const int q4 = lane >> 3;
     const int cur = c;
     if (lane == 0) c = atomicAdd(work, 1);
+    auto put = [&](double x) {
+      reinterpret_cast<double*>(q4 < 2 ? f.AT : f.AN)[2 * n + (q4 & 1)] = x;
+      if (f.AT32) reinterpret_cast<float*>(q4 < 2 ? f.AT32 : f.AN32)[2 * n + (q4 & 1)] = static_cast<float>(x);
+    };
     if (cd.count == 1) {
-      if (lane == 0) {
-        f.AT[n] = make_double2(v.x, v.y);
-        f.AN[n] = make_double2(v.z, v.w);
-        if (f.AT32) {
-          f.AT32[n] = make_float2(static_cast<float>(v.x), static_cast<float>(v.y));
-          f.AN32[n] = make_float2(static_cast<float>(v.z), static_cast<float>(v.w));
-        }
-      }
+      if (mine) put(v);
       continue;
     }
-    int prev = 0;
-    if (lane == 0) {
-      f.partial[cur] = v;
+    if (mine) {
+      reinterpret_cast<double*>(f.partial + cur)[q4] = v;
       __threadfence();
-      prev = atomicAdd(f.counter + n, 1);
     }
+    __syncwarp();
+    int prev = 0;
+    if (lane == 0) prev = atomicAdd(f.counter + n, 1);
     prev = __shfl_sync(0xffffffffu, prev, 0);
     if (prev == cd.count - 1) {
       __threadfence();
@@ -911,16 +911,9 @@ __global__ void __launch_bounds__(kHistThreads)
         r.z += p1.x;
         r.w += p1.y;
       }
-      r = make_double4(warp_sum(r.x), warp_sum(r.y), warp_sum(r.z), warp_sum(r.w));
-      if (lane == 0) {
-        f.AT[n] = make_double2(r.x, r.y);
-        f.AN[n] = make_double2(r.z, r.w);
-        if (f.AT32) {
-          f.AT32[n] = make_float2(static_cast<float>(r.x), static_cast<float>(r.y));
-          f.AN32[n] = make_float2(static_cast<float>(r.z), static_cast<float>(r.w));
-        }
-        f.counter[n] = 0;
-      }
+      const double s = warp_reduce4<double>(r.x, r.y, r.z, r.w);
+      if (mine) put(s);
+      if (lane == 0) f.counter[n] = 0;
     }
   }
 }
