@@ -213,6 +213,54 @@ __device__ __forceinline__ void assemble_pair32(const DevFault<float>& f, int m,
   *Yc = make_float2(tr + si, -ti + sr);
 }
 
+// The same per-mode inputs and pair assembly in FP64.
+struct ModeIn64 {
+  double2 D, K, AT, AN, C;
+};
+
+__device__ __forceinline__ ModeIn64 load_mode_in(const DevFault<double>& f, int m, int m_dt, double dt) {
+  ModeIn64 in;
+  in.D = f.dhat[m];
+  in.K = f.khat[m];
+  in.AT = f.AT[m];
+  in.AN = f.AN[m];
+  double w0T = 0.0, w0N = 0.0;
+  if ((m_dt & (m_dt - 1)) == 0) {
+    const double2 w0 = f.w0pow[static_cast<size_t>(m) * kPow2Slots + (31 - __clz(m_dt))];
+    w0T = w0.x;
+    w0N = w0.y;
+  } else {
+    const int lim = min(m_dt, f.Mn[m]);
+    for (int j = 0; j < lim; ++j) {
+      const double2 w = f.w[f.w_off[m] + j];
+      w0T += w.x;
+      w0N += w.y;
+    }
+  }
+  // S dt and mu w0 nearly cancel (C(k, 0) = -(1 - r^2)): their sum first
+  in.C = make_double2(f.S * dt + f.mu * w0T, f.S * dt + f.mu * w0N);
+  return in;
+}
+
+__device__ __forceinline__ void assemble_pair64(const DevFault<double>& f, int m, double k, double2 Zm, double2 Zc,
+                                                const ModeIn64& in, double2* U, double2* Q, double2* Ym, double2* Yc) {
+  const int half = f.N >> 1;
+  *U = make_double2(0.5 * (Zm.x + Zc.x), 0.5 * (Zm.y - Zc.y));
+  *Q = make_double2(0.5 * (Zm.y + Zc.y), 0.5 * (Zc.x - Zm.x));
+  double tr = 0.0, ti = 0.0, sr = 0.0, si = 0.0;
+  if (m > 0) {
+    tr = -k * (f.S * in.D.x + in.C.x * U->x + f.mu * in.AT.x);
+    if (m < half) {
+      // the Nyquist coefficient of a real sequence is real
+      ti = -k * (f.S * in.D.y + in.C.x * U->y + f.mu * in.AT.y);
+      sr = f.S * in.K.y + in.C.y * Q->y + f.mu * in.AN.y;
+      si = -(f.S * in.K.x + in.C.y * Q->x + f.mu * in.AN.x);
+    }
+  }
+  *Ym = make_double2(tr - si, ti + sr);
+  *Yc = make_double2(tr + si, sr - ti);
+}
+
 // Precision-form assembly of one coefficient n of the full spectrum (the
 // four-step passes): the pair (m, N-m), m = min(n, N-n), in FP32 from the
 // FP32 per-mode inputs, Y[n] its half; U, Q of mode m are kept (pass 2) by
@@ -323,6 +371,21 @@ __device__ __forceinline__ float2 f2sub(float2 a, float2 b) { return make_float2
 __device__ __forceinline__ float2 f2mul(float2 a, float2 b) {
   return make_float2(fmaf(a.x, b.x, -a.y * b.y), fmaf(a.x, b.y, a.y * b.x));
 }
+__device__ __forceinline__ double2 f2add(double2 a, double2 b) { return make_double2(a.x + b.x, a.y + b.y); }
+__device__ __forceinline__ double2 f2sub(double2 a, double2 b) { return make_double2(a.x - b.x, a.y - b.y); }
+__device__ __forceinline__ double2 f2mul(double2 a, double2 b) {
+  return make_double2(fma(a.x, b.x, -a.y * b.y), fma(a.x, b.y, a.y * b.x));
+}
+// v times -i sg (a quarter turn; sg = +1 forward, -1 inverse) and the other
+// eighth turns follow; the sign of an FP64 product is flipped on the integer
+// pipe (the FP64 pipe is scarce).
+__device__ __forceinline__ double flip(double v, double sg) {
+  return __longlong_as_double(__double_as_longlong(v) ^ (__double_as_longlong(sg) & (1LL << 63)));
+}
+__device__ __forceinline__ float flip(float v, float sg) { return sg * v; }
+__device__ __forceinline__ double2 quarter(double2 v, double sg) {
+  return make_double2(flip(v.y, sg), flip(v.x, -sg));
+}
 
 // v * w8^K with w8 = exp(-sg 2 pi i / 8): sg = +1 forward, -1 inverse
 // (one code path for both directions keeps the kernels small)
@@ -336,9 +399,18 @@ __device__ __forceinline__ float2 rot8(float2 v, float sg) {
   return v;
 }
 
+// Eighth turns of an FP64 value (the radix-4 and radix-2 stages use quarter
+// turns only).
 template <int K>
-__device__ __forceinline__ void bfly(float2& a, float2& b, float sg) {
-  const float2 s = f2add(a, b), d = f2sub(a, b);
+__device__ __forceinline__ double2 rot8(double2 v, double sg) {
+  static_assert(K == 0 || K == 2, "radix-4 stages");
+  if constexpr (K == 0) return v;
+  return quarter(v, sg);
+}
+
+template <int K, class C, class S>
+__device__ __forceinline__ void bfly(C& a, C& b, S sg) {
+  const C s = f2add(a, b), d = f2sub(a, b);
   a = s;
   b = rot8<K>(d, sg);
 }
@@ -367,15 +439,28 @@ __device__ __forceinline__ void dft8(float2 (&v)[8], float sg) {
   v[6] = t;
 }
 
-template <int O, int E>
-__device__ __forceinline__ void dft4(float2 (&v)[E], float sg) {
+template <int O, int E, class C, class S>
+__device__ __forceinline__ void dft4(C (&v)[E], S sg) {
   bfly<0>(v[O + 0], v[O + 2], sg);
   bfly<2>(v[O + 1], v[O + 3], sg);
   bfly<0>(v[O + 0], v[O + 1], sg);
   bfly<0>(v[O + 2], v[O + 3], sg);
-  const float2 t = v[O + 1];
+  const C t = v[O + 1];
   v[O + 1] = v[O + 2];
   v[O + 2] = t;
+}
+
+// w_N^a from the N/2-entry table (a < N), conjugated for the inverse
+__device__ __forceinline__ float2 tw_full(const float2* tw, int a, int half, bool inv) {
+  float2 w = a < half ? tw[a] : make_float2(-tw[a - half].x, -tw[a - half].y);
+  if (inv) w.y = -w.y;
+  return w;
+}
+
+__device__ __forceinline__ double2 tw_full(const double2* tw, int a, int half, bool inv) {
+  const double2 w = tw[a < half ? a : a - half];
+  const double sa = a < half ? 1.0 : -1.0;
+  return make_double2(flip(w.x, sa), flip(w.y, inv ? -sa : sa));
 }
 
 // One Stockham stage over buf (length L = 2^LGL, L/EPT threads holding EPT
@@ -385,8 +470,9 @@ __device__ __forceinline__ void dft4(float2 (&v)[E], float sg) {
 // A[(j - k) R + k + r Ns] = V_r (self-sorting; natural order after the last
 // stage).  Twiddles come from the L/2-entry table exp(-2 pi i a / L); all
 // index arithmetic is shifts and masks of compile-time sizes.
-template <int R, int LGL, int EPT = 8>
-__device__ __forceinline__ void stockham_stage(float2* buf, const float2* tw, int lgNs, int tid, float sg) {
+// MASK: only the threads with `on` transform, the others pass the barriers.
+template <int R, int LGL, int EPT = 8, bool MASK = false, class C, class S>
+__device__ __forceinline__ void stockham_stage(C* buf, const C* tw, int lgNs, int tid, S sg, bool on = true) {
   constexpr int L = 1 << LGL;
   constexpr int NB = EPT / R;  // butterflies per thread
   constexpr int LGR = R == 8 ? 3 : (R == 4 ? 2 : 1);
@@ -394,7 +480,8 @@ __device__ __forceinline__ void stockham_stage(float2* buf, const float2* tw, in
   constexpr int stride = L / R;
   constexpr int half = L >> 1;
   const int Ns = 1 << lgNs;
-  float2 v[EPT];
+  C v[EPT];
+  if (!MASK || on) {
 #pragma unroll
   for (int q = 0; q < NB; ++q) {
     const int j = tid + q * nth;
@@ -402,11 +489,13 @@ __device__ __forceinline__ void stockham_stage(float2* buf, const float2* tw, in
     const int tstep = k << (LGL - lgNs - LGR);
 #pragma unroll
     for (int r = 0; r < R; ++r) {
-      float2 x = buf[j + r * stride];
+      C x = buf[j + r * stride];
       if (r > 0) {
         const int a = r * tstep;
-        float2 w = a < half ? tw[a] : make_float2(-tw[a - half].x, -tw[a - half].y);
-        w.y *= sg;
+        C w;
+        if constexpr (sizeof(S) == 4) w = a < half ? tw[a] : make_float2(-tw[a - half].x, -tw[a - half].y);
+        else w = tw_full(tw, a, half, false);
+        w.y = flip(w.y, sg);
         x = f2mul(x, w);
       }
       v[q * R + r] = x;
@@ -421,7 +510,9 @@ __device__ __forceinline__ void stockham_stage(float2* buf, const float2* tw, in
 #pragma unroll
     for (int q = 0; q < EPT / 2; ++q) bfly<0>(v[2 * q], v[2 * q + 1], sg);
   }
+  }
   __syncthreads();
+  if (!MASK || on) {
 #pragma unroll
   for (int q = 0; q < NB; ++q) {
     const int j = tid + q * nth;
@@ -430,14 +521,15 @@ __device__ __forceinline__ void stockham_stage(float2* buf, const float2* tw, in
 #pragma unroll
     for (int r = 0; r < R; ++r) buf[base + r * Ns] = v[q * R + r];
   }
+  }
   __syncthreads();
 }
 
 // FFT of length 2^LGL in buf: sg = +1 forward, -1 unscaled inverse.
 // EPT = 8: radix-8 stages (+4 or 2); EPT = 4: radix-4 stages (+2), twice
 // the threads for the same length.
-template <int LGL, int EPT = 8>
-__device__ __noinline__ void fft_r8(float2* buf, const float2* tw, int tid, float sg) {
+template <int LGL, int EPT = 8, bool MASK = false, class C, class S>
+__device__ __noinline__ void fft_r8(C* buf, const C* tw, int tid, S sg, bool on = true) {
   if constexpr (EPT == 8) {
 #pragma unroll 1
     for (int s = 0; s < LGL / 3; ++s) stockham_stage<8, LGL>(buf, tw, 3 * s, tid, sg);
@@ -445,8 +537,8 @@ __device__ __noinline__ void fft_r8(float2* buf, const float2* tw, int tid, floa
     if constexpr (LGL % 3 == 1) stockham_stage<2, LGL>(buf, tw, 3 * (LGL / 3), tid, sg);
   } else {
 #pragma unroll 1
-    for (int s = 0; s < LGL / 2; ++s) stockham_stage<4, LGL, 4>(buf, tw, 2 * s, tid, sg);
-    if constexpr (LGL % 2 == 1) stockham_stage<2, LGL, 4>(buf, tw, 2 * (LGL / 2), tid, sg);
+    for (int s = 0; s < LGL / 2; ++s) stockham_stage<4, LGL, 4, MASK>(buf, tw, 2 * s, tid, sg, on);
+    if constexpr (LGL % 2 == 1) stockham_stage<2, LGL, 4, MASK>(buf, tw, 2 * (LGL / 2), tid, sg, on);
   }
 }
 
@@ -565,13 +657,6 @@ __device__ __forceinline__ int seq_row(int q, int N2) {
   if (q == 1) return N2 >> 1;
   return (q & 1) ? N2 - (q >> 1) : (q >> 1);
 }
-// w_N^a from the N/2-entry table (a < N), conjugated for the inverse
-__device__ __forceinline__ float2 tw_full(const float2* tw, int a, int half, bool inv) {
-  float2 w = a < half ? tw[a] : make_float2(-tw[a - half].x, -tw[a - half].y);
-  if (inv) w.y = -w.y;
-  return w;
-}
-
 __device__ __forceinline__ void cluster_arrive_relaxed() {
   asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
 }
@@ -591,12 +676,21 @@ __device__ __forceinline__ uint32_t cluster_map(const void* p, unsigned rank) {
 __device__ __forceinline__ void st_cluster(uint32_t addr, float2 v) {
   asm volatile("st.shared::cluster.v2.f32 [%0], {%1, %2};" ::"r"(addr), "f"(v.x), "f"(v.y) : "memory");
 }
+__device__ __forceinline__ void st_cluster(uint32_t addr, double2 v) {
+  asm volatile("st.shared::cluster.v2.f64 [%0], {%1, %2};" ::"r"(addr), "d"(v.x), "d"(v.y) : "memory");
+}
 
 // Transforms of length 2^LGL (2^LGL/EPT threads each) side by side in buf.
-template <int LGL, int EPT>
-__device__ __forceinline__ void fft_r8_batch(float2* buf, const float2* tw, int tid, float sg) {
+template <int LGL, int EPT, class C, class S>
+__device__ __forceinline__ void fft_r8_batch(C* buf, const C* tw, int tid, S sg) {
   constexpr int per = (1 << LGL) / EPT;
   fft_r8<LGL, EPT>(buf + (tid / per) * (1 << LGL), tw, tid % per, sg);
+}
+// The same by the first `nth` threads of a larger CTA.
+template <int LGL, int EPT, class C, class S>
+__device__ __forceinline__ void fft_r8_masked(C* buf, const C* tw, int tid, S sg, int nth) {
+  constexpr int per = (1 << LGL) / EPT;
+  fft_r8<LGL, EPT, true>(buf + (tid / per) * (1 << LGL), tw, tid % per, sg, tid < nth);
 }
 
 template <int LGN, int EPT, int CC>
@@ -738,6 +832,132 @@ __global__ void __launch_bounds__(CGeom<LGN, EPT, batch_cluster_ctas(1 << LGN)>:
   constexpr int CC = batch_cluster_ctas(1 << LGN);
   const DevFault<float>& f = fs[blockIdx.x / CC];
   spectral_cluster_body<LGN, EPT, CC>(f, pass, m_dt, m_dt * f.dt_min);
+}
+
+// The FP64 pass of a small fault on a cluster: the same four-step transform,
+// inputs and assembly in FP64 (N <= kCluster64MaxN).  One SM's FP64 pipe (2
+// operations a clock) would take 15 us over the transforms of N = 512 alone,
+// so even the smallest faults are spread over as many CTAs as keep a row and
+// its mirror together (two rows a CTA); four kernels a pass had cost a launch
+// and two memory latencies each (figures at kCluster64MaxN).  The
+// status word is read once per thread: where a step has failed nothing is
+// written (no early exit, the barriers need every CTA).
+__host__ __device__ constexpr int cluster64_ctas(int N) {
+  int lg = 0;
+  while ((1 << lg) < N) ++lg;
+  const int N1 = 1 << (lg / 2), N2 = 1 << (lg - lg / 2);
+  const int c = N1 < N2 / 2 ? N1 : N2 / 2;
+  return c < 16 ? c : 16;
+}
+
+template <int LGN>
+__device__ __forceinline__ void spectral_cluster64_body(const DevFault<double>& f, int pass, int m_dt, double dt) {
+  using G = CGeom<LGN, 4, cluster64_ctas(1 << LGN)>;
+  const unsigned c = cluster_rank();
+  constexpr int N = G::N, half = N >> 1, nth = G::nth, EPT = 4;
+  constexpr int per = N / G::C;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  double2* colbuf = reinterpret_cast<double2*>(smem_raw);  // [cols][N2]
+  double2* rowbuf = colbuf + per;                           // [rows][N1]
+  double2* twc = rowbuf + per;
+  double2* twr = twc + (G::N2 >> 1);
+  // one thread an element: every global load of the pass is in flight at
+  // once, one latency; the transforms run on the first nth threads (4 values
+  // each a stage)
+  const int e = threadIdx.x;
+  const bool el = e < per;
+  const int n1_0 = static_cast<int>(c) * G::cols;
+  const int q0 = static_cast<int>(c) * G::rows;
+  cluster_arrive_relaxed();
+  pdl_trigger();
+  // as a column element: column b, index k2 (= n2 of the input); as a row
+  // element: row k2r of the pair-adjacent sequence, index k1 (= n1)
+  const int b = e / G::N2, k2 = e % G::N2;
+  const int k2r = seq_row(q0 + e / G::N1, G::N2), k1 = e % G::N1;
+  const int m = k2r + G::N2 * k1;
+  const int ein = (e % G::cols) * G::N2 + e / G::cols;                // where the input and output element sits
+  const int nin = (n1_0 + e % G::cols) + G::N1 * (e / G::cols);
+  const bool lead = el && m <= half;
+  double2 wf = make_double2(0.0, 0.0), wi = wf;
+  ModeIn64 mi{};
+  unsigned failed;
+  {
+    // static inputs and the previous commit's before the wait; V1 (pass 2)
+    // and the status word behind the pass-1 Newton
+    double v = 0.0, kap = 0.0;
+    double2 tc = wf, tr = wf;
+    if (e < (G::N2 >> 1)) tc = f.tw[e * G::N1];
+    if (e < (G::N1 >> 1)) tr = f.tw[e * G::N2];
+    if (el) {
+      v = f.V[nin];
+      kap = f.kappa[nin];
+      wf = tw_full(f.tw, (n1_0 + b) * k2, half, false);
+      wi = tw_full(f.tw, k1 * k2r, half, true);
+    }
+    if (lead) mi = load_mode_in(f, m, m_dt, dt);
+    pdl_wait();
+    failed = *f.status;
+    reset_newton_stats(f, pass, c == 0 && e == 0);
+    if (el && pass != 1) v = 0.5 * (v + f.V1[nin]);
+    if (e < (G::N2 >> 1)) twc[e] = tc;
+    if (e < (G::N1 >> 1)) twr[e] = tr;
+    if (el) colbuf[ein] = make_double2(v, kap * v);
+  }
+  const double kunit = kTwoPi / f.L;
+  __syncthreads();
+  fft_r8_masked<G::lg2, EPT>(colbuf, twc, e, 1.0, nth);
+  cluster_wait();
+  if (el) {
+    const int sq = row_seq(k2, G::N2);
+    st_cluster(cluster_map(rowbuf + (sq % G::rows) * G::N1 + n1_0 + b, static_cast<unsigned>(sq / G::rows)),
+               f2mul(colbuf[e], wf));
+  }
+  cluster_arrive();
+  cluster_wait();
+  fft_r8_masked<G::lg1, EPT>(rowbuf, twr, e, 1.0, nth);
+  if (lead) {
+    const int k2p = (k2r == 0 || k2r == (G::N2 >> 1)) ? k2r : G::N2 - k2r;
+    const int k1p = k2r == 0 ? (G::N1 - k1) & (G::N1 - 1) : G::N1 - 1 - k1;
+    const int ep = (row_seq(k2p, G::N2) - q0) * G::N1 + k1p;
+    double2 U, Q, Ym, Yc;
+    assemble_pair64(f, m, kunit * m, rowbuf[e], rowbuf[ep], mi, &U, &Q, &Ym, &Yc);
+    if (pass == 2 && !failed) {
+      f.U2[m] = U;
+      f.Q2[m] = Q;
+    }
+    rowbuf[e] = Ym;
+    if (ep != e) rowbuf[ep] = Yc;
+  }
+  __syncthreads();
+  fft_r8_masked<G::lg1, EPT>(rowbuf, twr, e, -1.0, nth);
+  if (el)
+    st_cluster(cluster_map(colbuf + (k1 % G::cols) * G::N2 + k2r, static_cast<unsigned>(k1 / G::cols)),
+               f2mul(rowbuf[e], wi));
+  cluster_arrive();
+  cluster_wait();
+  fft_r8_masked<G::lg2, EPT>(colbuf, twc, e, -1.0, nth);
+  if (failed || !el) return;
+  constexpr double scale = 1.0 / N;
+  const double2 y = colbuf[ein];
+  f.y[nin] = make_double2(y.x * scale, y.y * scale);
+}
+
+// Threads of a CTA: one an element, a warp at least.
+__host__ __device__ constexpr int cluster64_threads(int N) {
+  return N / cluster64_ctas(N) > 32 ? N / cluster64_ctas(N) : 32;
+}
+
+template <int LGN>
+__global__ void __launch_bounds__(cluster64_threads(1 << LGN))
+    k_spectral_cluster64(const __grid_constant__ DevFault<double> f, int pass, int m_dt, double dt) {
+  spectral_cluster64_body<LGN>(f, pass, m_dt, dt);
+}
+
+template <int LGN>
+__global__ void __launch_bounds__(cluster64_threads(1 << LGN))
+    k_spectral_cluster64_b(const DevFault<double>* __restrict__ fs, int pass, int m_dt) {
+  const DevFault<double>& f = fs[blockIdx.x / cluster64_ctas(1 << LGN)];
+  spectral_cluster64_body<LGN>(f, pass, m_dt, m_dt * f.dt_min);
 }
 
 // Row pass: for k2 in this CTA's B rows, transform t[k2 N1 + n1] over n1
@@ -2268,6 +2488,14 @@ static void with_lgn(int N, F&& fn) {
 }
 static_assert(kFusedMaxN == 1 << 14 && kClusterMinN == 1 << 11, "with_lgn covers the one-launch pass sizes");
 
+static size_t cluster64_smem(int N) {
+  int lg = 0;
+  while ((1 << lg) < N) ++lg;
+  const int N1 = 1 << (lg / 2), N2 = 1 << (lg - lg / 2);
+  const size_t per = static_cast<size_t>(N / cluster64_ctas(N));
+  return (2 * per + N1 / 2 + N2 / 2) * sizeof(double2);
+}
+
 // Launch with the attributes of the pass kernels: a cluster of `cluster`
 // CTAs (> 1), programmatic dependent launch behind the stream's previous
 // kernel (early; the kernel waits in pdl_wait()), and an event that fires
@@ -2341,6 +2569,19 @@ void launch_spectral(const DevFault<R>& f, int pass, int m_dt, cudaStream_t st, 
         } else {
           launch_attr(k_spectral_fused<LG>, dim3(1), dim3(f.N / 8), fused_smem(f.N), st, 1, pass == 2, started, f,
                       pass, m_dt, dt);
+        }
+      });
+      return;
+    }
+  }
+  if constexpr (sizeof(R) == 8) {
+    if (f.N <= kCluster64MaxN) {
+      with_lgn(f.N, [&](auto lg) {
+        constexpr int LG = decltype(lg)::value;
+        if constexpr ((1 << LG) <= kCluster64MaxN) {
+          constexpr int C = cluster64_ctas(1 << LG);
+          launch_attr(k_spectral_cluster64<LG>, dim3(C), dim3(cluster64_threads(f.N)), cluster64_smem(f.N), st, C, pass == 2,
+                      started, f, pass, m_dt, dt);
         }
       });
       return;
@@ -2578,6 +2819,20 @@ void launch_pass_batch(const FftGeom& g, const DevFault<R>* fs, int members, int
       return;
     }
   }
+  if constexpr (sizeof(R) == 8) {
+    if (N <= kCluster64MaxN) {
+      with_lgn(N, [&](auto lg) {
+        constexpr int LG = decltype(lg)::value;
+        if constexpr ((1 << LG) <= kCluster64MaxN) {
+          constexpr int C = cluster64_ctas(1 << LG);
+          launch_attr(k_spectral_cluster64_b<LG>, dim3(C * members), dim3(cluster64_threads(N)), cluster64_smem(N), st, C,
+                      false, static_cast<cudaEvent_t>(nullptr), fs, pass, m_dt);
+        }
+      });
+      k_newton_b<R><<<dim3((N + 31) / 32, members), 32, 0, st>>>(fs, pass, m_dt);
+      return;
+    }
+  }
   const size_t cs = col_smem<R>(g), rs = row_smem<R>(g);
   const dim3 gc(g.N1 / g.Bc, members), gr(g.N2 / g.Br, members);
   k_col_b<R, false, PRO_PASS><<<gc, g.tc, cs, st>>>(g, fs, pass, m_dt);
@@ -2604,6 +2859,16 @@ void configure_batch_kernels(const FftGeom& g) {
           cudaFuncSetAttribute(k_spectral_cluster_b<LG, kClusterEPT>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
         } else {
           allow_smem(k_spectral_fused_b<LG>, fused_smem(g.N));
+        }
+      });
+  }
+  if constexpr (sizeof(R) == 8) {
+    if (g.N <= kCluster64MaxN)
+      with_lgn(g.N, [&](auto lg) {
+        constexpr int LG = decltype(lg)::value;
+        if constexpr ((1 << LG) <= kCluster64MaxN) {
+          allow_smem(k_spectral_cluster64_b<LG>, cluster64_smem(g.N));
+          cudaFuncSetAttribute(k_spectral_cluster64_b<LG>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
         }
       });
   }
@@ -2784,6 +3049,16 @@ void configure_kernels(const FftGeom& g) {
           cudaFuncSetAttribute(k_spectral_cluster<LG, kClusterEPT>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
         } else {
           allow_smem(k_spectral_fused<LG>, fused_smem(g.N));
+        }
+      });
+  }
+  if constexpr (sizeof(R) == 8) {
+    if (g.N <= kCluster64MaxN)
+      with_lgn(g.N, [&](auto lg) {
+        constexpr int LG = decltype(lg)::value;
+        if constexpr ((1 << LG) <= kCluster64MaxN) {
+          allow_smem(k_spectral_cluster64<LG>, cluster64_smem(g.N));
+          cudaFuncSetAttribute(k_spectral_cluster64<LG>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
         }
       });
   }

@@ -153,6 +153,11 @@ struct DevFault {
 constexpr int kFusedMaxN = 16384;
 constexpr int kClusterMinN = 2048;
 constexpr int kClusterCTAs = 8;
+// One-launch FP64 spectral pass up to this N (a cluster of up to 16 CTAs;
+// quasi-dynamic steps of two passes, one launch against four: N = 256 39
+// against 62 us, 4096 53 against 82 us, 8192 62 against 86 us; above it the
+// 16 SMs' FP64 pipes are slower than every SM's).
+constexpr int kCluster64MaxN = 8192;
 // CTAs per cluster for a given N: 16 (a non-portable cluster size) from
 // N = 4096: half the work per CTA on the latency-bound pass (flushed steps
 // without history at N = 4096: 35.3 -> 33.0 us; N = 8192: 49.2 -> 36.9 us;
