@@ -132,8 +132,14 @@ struct sbiem_s {
   long long* snap_steps = nullptr;
   void* tune_slots = nullptr;   // one ring slot per mode (the autotuner's timed steps)
   void* undo = nullptr;          // ring-sized
-  double* dfull = nullptr;
-  double* d_err = nullptr;
+  double* dfull = nullptr;       // slip of the whole trial step
+  // the whole step's staging (sbiem_run advances it beside the first half
+  // step): descriptors that differ from f64 / f32 in the buffers a pass writes
+  DevFault<double> trial64{};
+  DevFault<float> trial32{};
+  unsigned long long* trial_work = nullptr;
+  TrialReport* h_trial = nullptr;  // page-locked
+  cudaEvent_t ev_sums = nullptr, ev_trial = nullptr;
   MlpDev* mlp = nullptr;         // deployed Newton initial-guess network
   float* harvest = nullptr;
   unsigned long long* harvest_count = nullptr;
@@ -215,6 +221,9 @@ void free_all(sbiem_s* s) {
   if (s->ev_fork) cudaEventDestroy(s->ev_fork);
   if (s->ev_join) cudaEventDestroy(s->ev_join);
   if (s->ev_started) cudaEventDestroy(s->ev_started);
+  for (cudaEvent_t e : {s->ev_sums, s->ev_trial})
+    if (e) cudaEventDestroy(e);
+  if (s->h_trial) cudaFreeHost(s->h_trial);
 }
 
 bool is_pow2(int64_t n) { return n > 0 && (n & (n - 1)) == 0; }
@@ -480,27 +489,14 @@ void enqueue_step_lag_t(sbiem_s* s, const DevFault<R>& f, int m, cudaStream_t st
   launch_commit<R>(f, m, st, p);
 }
 
-// The step without its commit: pass-2 results stay staged (delta2, V2, ...).
-template <class R>
-void enqueue_trial_t(sbiem_s* s, const DevFault<R>& f, int m, cudaStream_t st) {
-  launch_history<R>(f, m, s->hist_grid, st);
-  launch_pass<R>(f, 1, m, st);
-  launch_pass<R>(f, 2, m, st);
-}
-
 void enqueue_step(sbiem_s* s, int m, cudaStream_t st) {
   if (s->fp32()) enqueue_step_t<float>(s, s->f32, m, st);
   else enqueue_step_t<double>(s, s->f64, m, st);
 }
 
-void enqueue_trial(sbiem_s* s, int m, cudaStream_t st) {
-  if (s->fp32()) enqueue_trial_t<float>(s, s->f32, m, st);
-  else enqueue_trial_t<double>(s, s->f64, m, st);
-}
-
-void ring_undo(sbiem_s* s, int m, int dir) {
-  if (s->fp32()) launch_ring_undo<float>(s->f32, m, s->undo, dir, s->stream);
-  else launch_ring_undo<double>(s->f64, m, s->undo, dir, s->stream);
+void ring_undo(sbiem_s* s, int m, int dir, cudaStream_t st) {
+  if (s->fp32()) launch_ring_undo<float>(s->f32, m, s->undo, dir, st);
+  else launch_ring_undo<double>(s->f64, m, s->undo, dir, st);
 }
 
 // Device buffers of the state snapshot (allocated on first use).
@@ -516,30 +512,88 @@ bool ensure_snapshot(sbiem_s* s) {
 }
 
 // Save (save = true) or restore the committed state that a step changes.
-int snapshot(sbiem_s* s, bool save) {
-  auto& f = s->f64;
-  const size_t nb = sizeof(double) * s->N;
-  double* arrs[] = {f.V, f.xV, f.psi, f.thd, f.delta, f.th};
-  for (int k = 0; k < 6; ++k) {
-    double* sn = s->snap + static_cast<size_t>(k) * s->N;
-    CK(cudaMemcpyAsync(save ? sn : arrs[k], save ? arrs[k] : sn, nb, cudaMemcpyDeviceToDevice, s->stream));
+int snapshot(sbiem_s* s, bool save, cudaStream_t st) {
+  const Snapshot sn{s->snap, s->snap_spec, s->snap_head, s->snap_steps};
+  if (s->fp32()) launch_snapshot<float>(s->f32, sn, save ? 0 : 1, st);
+  else launch_snapshot<double>(s->f64, sn, save ? 0 : 1, st);
+  CK(cudaGetLastError());
+  return SBIEM_OK;
+}
+
+// Staging of the whole trial step of sbiem_run, beside the handle's own.
+template <class R>
+bool trial_buffers(sbiem_s* s, const DevFault<R>& f, DevFault<R>& t) {
+  bool ok = true;
+  t = f;
+  for (double** d : {&t.V1, &t.thd1, &t.x1, &t.V2, &t.x2, &t.psi2, &t.th2, &t.thd2}) *d = alloc_n<double>(s, s->N, &ok);
+  t.delta2 = s->dfull;
+  for (Cx<R>** c : {&t.Z, &t.zt, &t.y}) *c = alloc_n<Cx<R>>(s, s->N, &ok);
+  if constexpr (sizeof(R) == 4) {
+    t.zin2 = alloc_n<float2>(s, s->N, &ok);
+    for (float2** c : {&t.U2f, &t.Q2f, &t.AT32, &t.AN32}) *c = alloc_n<float2>(s, s->nmodes, &ok);
+    for (double2** c : {&t.AT, &t.AN}) *c = alloc_n<double2>(s, s->nmodes, &ok);
+  } else {
+    for (double2** c : {&t.U2, &t.Q2}) *c = alloc_n<double2>(s, s->nmodes, &ok);
+    // the whole step's sums are what the second half step's lack its newest
+    // slot of: the overlapped form's BT/BN
+    t.AT = f.BT;
+    t.AN = f.BN;
   }
-  double* snt = s->snap + static_cast<size_t>(6) * s->N;
-  CK(cudaMemcpyAsync(save ? snt : f.t, save ? f.t : snt, sizeof(double), cudaMemcpyDeviceToDevice, s->stream));
-  const size_t sb = sizeof(double2) * s->nmodes;
-  CK(cudaMemcpyAsync(save ? s->snap_spec : f.dhat, save ? f.dhat : s->snap_spec, sb, cudaMemcpyDeviceToDevice, s->stream));
-  CK(cudaMemcpyAsync(save ? s->snap_spec + s->nmodes : f.khat, save ? f.khat : s->snap_spec + s->nmodes, sb,
-                     cudaMemcpyDeviceToDevice, s->stream));
-  CK(cudaMemcpyAsync(save ? s->snap_head : f.head, save ? f.head : s->snap_head, sizeof(int32_t) * s->nmodes,
-                     cudaMemcpyDeviceToDevice, s->stream));
-  CK(cudaMemcpyAsync(save ? s->snap_steps : f.steps_done, save ? f.steps_done : s->snap_steps, sizeof(long long),
-                     cudaMemcpyDeviceToDevice, s->stream));
-  if (!save && f.dhat32) {
-    // the FP32 copies of the restored running sums
-    launch_to_float2(f.dhat, f.dhat32, s->nmodes, s->stream);
-    launch_to_float2(f.khat, f.khat32, s->nmodes, s->stream);
-  }
-  if (!save && s->f32.zin1) launch_zin(f.V, f.kappa, s->f32.zin1, s->N, s->stream);
+  t.it_sum = alloc_n<unsigned long long>(s, 1, &ok);
+  t.it_max = alloc_n<int>(s, 1, &ok);
+  return ok;
+}
+
+// One attempt of sbiem_run from the committed state, all of it enqueued: the
+// whole step of m (its staging apart, not committed) on the side stream beside
+// the first half step, then the second half step, then the report (eps, status)
+// to s->h_trial.  The state and the ring slots the half steps overwrite are
+// saved beside the sums.  A step that fails sets the status word: whatever
+// follows it commits nothing or is undone by the caller.
+// The second half step's sums: in FP64 those of the whole step plus the first
+// half step's slot, as in the overlapped form (the same lags in another
+// grouping); the FP32 form sweeps them anew, so that the sums round as those
+// of single steps do (at the start of a rupture the static and history terms
+// nearly cancel, and a regrouped FP32 sum moved the normal traction by 1e-4).
+template <class R>
+int enqueue_attempt(sbiem_s* s, const DevFault<R>& f, const DevFault<R>& staging, int m) {
+  const cudaStream_t st = s->stream, sd = s->side;
+  const int h = m / 2;
+  int p = 0;
+  while ((1 << p) < h) ++p;
+  // the handle as it is now, with the trial's staging
+  DevFault<R> t = f;
+#define STAGE(x) t.x = staging.x
+  STAGE(V1); STAGE(thd1); STAGE(x1); STAGE(V2); STAGE(x2); STAGE(psi2); STAGE(th2); STAGE(thd2); STAGE(delta2);
+  STAGE(Z); STAGE(zt); STAGE(y); STAGE(zin2); STAGE(U2f); STAGE(Q2f); STAGE(U2); STAGE(Q2);
+  STAGE(AT); STAGE(AN); STAGE(AT32); STAGE(AN32); STAGE(it_sum); STAGE(it_max);
+#undef STAGE
+  CK(cudaEventRecord(s->ev_fork, st));
+  CK(cudaStreamWaitEvent(sd, s->ev_fork, 0));
+  int rc = snapshot(s, true, sd);
+  if (rc) return rc;
+  ring_undo(s, m, 0, sd);
+  launch_history<R>(t, m, s->hist_grid, st);
+  CK(cudaEventRecord(s->ev_sums, st));
+  CK(cudaStreamWaitEvent(sd, s->ev_sums, 0));
+  launch_history<R>(f, h, s->hist_grid, st);
+  launch_pass<R>(t, 1, m, sd);
+  launch_pass<R>(t, 2, m, sd);
+  CK(cudaEventRecord(s->ev_trial, sd));
+  launch_pass<R>(f, 1, h, st);
+  launch_pass<R>(f, 2, h, st);
+  // the whole step has read the committed state, which is saved
+  CK(cudaStreamWaitEvent(st, s->ev_trial, 0));
+  constexpr bool lag = sizeof(R) == 8;
+  if (h > 1) launch_push_multi<R>(f, h, st);
+  launch_commit<R>(f, h, st, lag ? p : -1);
+  if (!lag) launch_history<R>(f, h, s->hist_grid, st);
+  launch_pass<R>(f, 1, h, st);
+  launch_pass<R>(f, 2, h, st);
+  if (h > 1) launch_push_multi<R>(f, h, st);
+  launch_commit<R>(f, h, st);
+  launch_trial_report(f.delta, s->dfull, s->N, f.status, s->trial_work, s->h_trial, st);
+  CK(cudaGetLastError());
   return SBIEM_OK;
 }
 
@@ -988,6 +1042,18 @@ int sbiem_status(sbiem_t s, uint32_t* flags, int64_t* steps_done, int clear) {
 
 namespace {
 
+// Synchronize and read the status word; a set one is cleared.
+int take_status(sbiem_s* s, uint32_t* st) {
+  CK(cudaMemcpyAsync(s->h_status, s->f64.status, sizeof(unsigned), cudaMemcpyDeviceToHost, s->stream));
+  CK(cudaStreamSynchronize(s->stream));
+  *st = *s->h_status;
+  if (*st) {
+    s->lag_m = -1;  // a rejected step left AT/AN of its start
+    CK(cudaMemsetAsync(s->f64.status, 0, sizeof(unsigned), s->stream));
+  }
+  return SBIEM_OK;
+}
+
 // The overlapped step graph of m dt_min (captured and instantiated once).
 int lag_graph(sbiem_s* s, int m) {
   if (s->lag_graphs.count(m)) return SBIEM_OK;
@@ -1039,15 +1105,13 @@ int sbiem_step(sbiem_t s, double dt) {
   int m;
   int rc = dt_to_m(s, dt, &m);
   if (rc) return rc;
-  uint32_t before;
-  rc = sbiem_status(s, &before, nullptr, 1);
-  if (rc) return rc;
+  CK(cudaMemsetAsync(s->f64.status, 0, sizeof(unsigned), s->stream));
   if (s->pslots) s->pcur = static_cast<int>(s->pcount++ % s->pslots);
   s->lag_m = -1;
   enqueue_step(s, m, s->stream);
   CK(cudaGetLastError());
   uint32_t st;
-  rc = sbiem_status(s, &st, nullptr, 1);
+  rc = take_status(s, &st);
   if (rc) return rc;
   rc = status_to_code(st);
   if (rc) return fail(rc, "step rejected; state left at the start of the step");
@@ -1167,9 +1231,13 @@ int sbiem_run(sbiem_t s, double t_end, double eps0, int64_t m0, int64_t m_max, i
   bool ok = ensure_snapshot(s);
   if (!s->undo) {
     s->dfull = alloc_n<double>(s, s->N, &ok);
-    s->d_err = alloc_n<double>(s, 1, &ok);
+    s->trial_work = alloc_n<unsigned long long>(s, 2, &ok);
+    ok = ok && (s->fp32() ? trial_buffers<float>(s, s->f32, s->trial32) : trial_buffers<double>(s, f, s->trial64));
+    for (cudaEvent_t* e : {&s->ev_sums, &s->ev_trial})
+      if (ok && !*e) ok = cudaEventCreateWithFlags(e, cudaEventDisableTiming) == cudaSuccess;
+    if (ok && !s->h_trial) ok = cudaMallocHost(&s->h_trial, sizeof(TrialReport)) == cudaSuccess;
     const size_t slot = s->fp32() ? sizeof(Slot32) : sizeof(Slot64);
-    s->undo = dev_alloc(s, slot * static_cast<size_t>(std::max<int64_t>(s->total_slots, 1)));
+    if (ok) s->undo = dev_alloc(s, slot * static_cast<size_t>(std::max<int64_t>(s->total_slots, 1)));
     if (!s->undo) ok = false;
   }
   if (!ok) return fail(SBIEM_ERR_NOMEM, "adaptive run: snapshot allocation failed");
@@ -1190,7 +1258,8 @@ int sbiem_run(sbiem_t s, double t_end, double eps0, int64_t m0, int64_t m_max, i
   while (t < t_end * (1.0 - 1e-15) && accepted < max_steps) {
     if (m == 1) {
       enqueue_step(s, 1, s->stream);
-      rc = sbiem_status(s, &st, nullptr, 1);
+      CK(cudaGetLastError());
+      rc = take_status(s, &st);
       if (rc) return rc;
       if (st) {
         rc = fail(SBIEM_ERR_DTMIN, "step failed at dt_min (status bits " + std::to_string(st) +
@@ -1207,30 +1276,17 @@ int sbiem_run(sbiem_t s, double t_end, double eps0, int64_t m0, int64_t m_max, i
       continue;
     }
     const int mi = static_cast<int>(m);
-    // full step, not committed
-    enqueue_trial(s, mi, s->stream);
-    rc = sbiem_status(s, &st, nullptr, 1);
+    rc = s->fp32() ? enqueue_attempt<float>(s, s->f32, s->trial32, mi) : enqueue_attempt<double>(s, f, s->trial64, mi);
     if (rc) return rc;
-    if (st) {
-      m /= 2;
-      continue;
-    }
-    CK(cudaMemcpyAsync(s->dfull, f.delta2, sizeof(double) * s->N, cudaMemcpyDeviceToDevice, s->stream));
-    rc = snapshot(s, true);
-    if (rc) return rc;
-    ring_undo(s, mi, 0);
-    enqueue_step(s, mi / 2, s->stream);
-    enqueue_step(s, mi / 2, s->stream);
-    launch_maxdiff(f.delta, s->dfull, s->N, s->d_err, s->stream);
-    double eps = 0.0;
-    CK(cudaMemcpyAsync(&eps, s->d_err, sizeof(double), cudaMemcpyDeviceToHost, s->stream));
-    rc = sbiem_status(s, &st, nullptr, 1);
-    if (rc) return rc;
+    CK(cudaStreamSynchronize(s->stream));
+    st = s->h_trial->status;
+    const double eps = s->h_trial->eps;
+    if (st) CK(cudaMemsetAsync(f.status, 0, sizeof(unsigned), s->stream));
     const double factor = eps > 0.0 ? 0.9 * std::cbrt(eps0 / eps) : HUGE_VAL;
     if (st || eps > eps0) {
-      rc = snapshot(s, false);
+      rc = snapshot(s, false, s->stream);
       if (rc) return rc;
-      ring_undo(s, mi, 1);
+      ring_undo(s, mi, 1, s->stream);
       int64_t mn = m / 2;
       if (!st)
         while (mn > 1 && static_cast<double>(mn) > factor * static_cast<double>(m)) mn /= 2;
@@ -1808,7 +1864,7 @@ int sbiem_tune(sbiem_t s, int reps, int32_t* shape_out, double* gen_out, int32_t
       }
       std::vector<float> tm;
       for (int k = 0; k <= reps; ++k) {
-        int rcs = snapshot(s, true);
+        int rcs = snapshot(s, true, s->stream);
         if (rcs) {
           cudaEventDestroy(e0);
           cudaEventDestroy(e1);
@@ -1820,7 +1876,7 @@ int sbiem_tune(sbiem_t s, int reps, int32_t* shape_out, double* gen_out, int32_t
         CK(cudaGraphLaunch(s->lag_graphs[1], s->stream));
         CK(cudaEventRecord(e1, s->stream));
         CK(cudaEventSynchronize(e1));
-        rcs = snapshot(s, false);
+        rcs = snapshot(s, false, s->stream);
         if (rcs) {
           cudaEventDestroy(e0);
           cudaEventDestroy(e1);

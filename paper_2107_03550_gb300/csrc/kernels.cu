@@ -2292,19 +2292,89 @@ void launch_slot_swap(const DevFault<R>& f, void* buf, int dir, cudaStream_t st)
 template void launch_slot_swap<double>(const DevFault<double>&, void*, int, cudaStream_t);
 template void launch_slot_swap<float>(const DevFault<float>&, void*, int, cudaStream_t);
 
-// max_i |a_i - b_i| into *out (one block).
-__global__ void k_maxdiff(const double* a, const double* b, int n, double* out) {
-  __shared__ double sh[32];
+// The committed state of a fault saved (dir 0) or put back (dir 1) in one
+// launch: six element arrays, time, step count, running spectra and ring
+// heads; putting back also renews the FP32 copies that are made from them.
+// (Eleven copies had cost a launch each.)
+template <class R>
+__global__ void k_snapshot(const __grid_constant__ DevFault<R> f, const Snapshot sn, int dir) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < f.N) {
+    double* const live[6] = {f.V, f.xV, f.psi, f.thd, f.delta, f.th};
+#pragma unroll
+    for (int k = 0; k < 6; ++k) {
+      double* s = sn.el + static_cast<size_t>(k) * f.N + i;
+      if (dir == 0) *s = live[k][i];
+      else live[k][i] = *s;
+    }
+    if (dir == 1 && f.zin1) {
+      const double v = sn.el[i];
+      f.zin1[i] = make_float2(static_cast<float>(v), static_cast<float>(f.kappa[i] * v));
+    }
+  }
+  if (i < f.nmodes) {
+    if (dir == 0) {
+      sn.spec[i] = f.dhat[i];
+      sn.spec[f.nmodes + i] = f.khat[i];
+      sn.head[i] = f.head[i];
+    } else {
+      const double2 D = sn.spec[i], K = sn.spec[f.nmodes + i];
+      f.dhat[i] = D;
+      f.khat[i] = K;
+      f.head[i] = sn.head[i];
+      if (f.dhat32) {
+        f.dhat32[i] = make_float2(static_cast<float>(D.x), static_cast<float>(D.y));
+        f.khat32[i] = make_float2(static_cast<float>(K.x), static_cast<float>(K.y));
+      }
+    }
+  }
+  if (i == 0) {
+    double* t = sn.el + static_cast<size_t>(6) * f.N;
+    if (dir == 0) {
+      *t = *f.t;
+      *sn.steps = *f.steps_done;
+    } else {
+      *f.t = *t;
+      *f.steps_done = *sn.steps;
+    }
+  }
+}
+
+template <class R>
+void launch_snapshot(const DevFault<R>& f, const Snapshot& sn, int dir, cudaStream_t st) {
+  const int n = f.N > f.nmodes ? f.N : f.nmodes;
+  k_snapshot<R><<<(n + 255) / 256, 256, 0, st>>>(f, sn, dir);
+}
+template void launch_snapshot<double>(const DevFault<double>&, const Snapshot&, int, cudaStream_t);
+template void launch_snapshot<float>(const DevFault<float>&, const Snapshot&, int, cudaStream_t);
+
+// Outcome of a trial step to page-locked host memory: out->eps = max_i |a_i -
+// b_i| (NaN differences do not count, as in fmax) and the status word.  The
+// CTAs' maxima meet in work[0] (the bits of a non-negative double order like
+// its value), the last CTA to arrive (work[1]) reports and clears both.
+__global__ void __launch_bounds__(256) k_trial_report(const double* a, const double* b, int n, const unsigned* status,
+                                                      unsigned long long* work, TrialReport* out) {
+  __shared__ double sh[8];
   double m = 0.0;
-  for (int i = threadIdx.x; i < n; i += blockDim.x) m = fmax(m, fabs(a[i] - b[i]));
+  for (int i = blockIdx.x * 256 + threadIdx.x; i < n; i += gridDim.x * 256) m = fmax(m, fabs(a[i] - b[i]));
   for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
   if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = m;
   __syncthreads();
-  if (threadIdx.x < 32) {
-    m = (threadIdx.x < (blockDim.x >> 5)) ? sh[threadIdx.x] : 0.0;
-    for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
-    if (threadIdx.x == 0) *out = m;
-  }
+  if (threadIdx.x != 0) return;
+  for (int w = 1; w < 8; ++w) m = fmax(m, sh[w]);
+  atomicMax(work, static_cast<unsigned long long>(__double_as_longlong(m)));
+  __threadfence();
+  if (atomicAdd(work + 1, 1ull) != gridDim.x - 1) return;
+  __threadfence();
+  out->eps = __longlong_as_double(static_cast<long long>(atomicExch(work, 0ull)));
+  work[1] = 0ull;
+  out->status = *status;
+}
+
+void launch_trial_report(const double* a, const double* b, int n, const unsigned* status, unsigned long long* work,
+                         TrialReport* out, cudaStream_t st) {
+  const int grid = n / 1024 < 1 ? 1 : (n / 1024 > 152 ? 152 : n / 1024);
+  k_trial_report<<<grid, 256, 0, st>>>(a, b, n, status, work, out);
 }
 
 // ------------------------------------------------------------- weights
@@ -2977,10 +3047,6 @@ __global__ void k_zin(const double* V, const double* kappa, float2* zin, int n) 
 
 void launch_zin(const double* V, const double* kappa, float2* zin, int n, cudaStream_t st) {
   k_zin<<<(n + 255) / 256, 256, 0, st>>>(V, kappa, zin, n);
-}
-
-void launch_maxdiff(const double* a, const double* b, int n, double* out, cudaStream_t st) {
-  k_maxdiff<<<1, 1024, 0, st>>>(a, b, n, out);
 }
 
 template <class R>

@@ -279,8 +279,23 @@ template <class R> void launch_ring_undo(const DevFault<R>& f, int m_dt, void* u
 // (FP32 when in_f32, else FP64), n slots.
 template <class R> void launch_set_ring(Slot<R>* ring, const void* hT, const void* hN, bool in_f32, int64_t n,
                                         int sm_count, cudaStream_t st);
-// *out = max_i |a_i - b_i|.
-void launch_maxdiff(const double* a, const double* b, int n, double* out, cudaStream_t st);
+// Buffers of a state snapshot (6 N + 1 doubles, 2 nmodes spectra, heads, step
+// count): saved (dir 0) or put back (dir 1).
+struct Snapshot {
+  double* el;
+  double2* spec;
+  int32_t* head;
+  long long* steps;
+};
+template <class R> void launch_snapshot(const DevFault<R>& f, const Snapshot& sn, int dir, cudaStream_t st);
+// max_i |a_i - b_i| and the status word to page-locked host memory (work: two
+// zeroed words of device memory, left zeroed).
+struct TrialReport {
+  double eps;
+  unsigned status, pad;
+};
+void launch_trial_report(const double* a, const double* b, int n, const unsigned* status, unsigned long long* work,
+                         TrialReport* out, cudaStream_t st);
 // Weights of every lag from the Chebyshev table: quadrature 0 midpoint,
 // 1 the integral over each interval.
 template <class R> void launch_weights(const DevFault<R>& f, const double* cheb, int npieces, int deg,

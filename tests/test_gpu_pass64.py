@@ -16,6 +16,10 @@ pytestmark = pytest.mark.gpu
 @pytest.mark.parametrize("N", [16, 32, 64, 128, 256, 512, 1024, 2048, 4096, 8192, 16384])
 def test_pass_matches_oracle_at_every_size(N):
     w = seamount_rupture(N=N)
+    # a slip rate that varies at every N (the workload's patch lies outside the
+    # shortest faults, whose shear traction would be rounding alone)
+    i = np.arange(N)
+    w.V_init = 1e-9 * np.exp(np.cos(2 * np.pi * i / N) + 0.5 * np.sin(6 * np.pi * i / N + 1.0))
     o, g = oracle_for(w, eta_w=0.0), gpu_for(w, eta_w=0.0)
     for m in (1, 3, 2):
         assert o.step(m) == 0
