@@ -55,10 +55,6 @@ namespace {
 constexpr int kDirectThreads = 512;
 constexpr int kDirectWarps = kDirectThreads / 32;
 constexpr int kDirectRegs = 88;
-// Shared memory carve-out of the sweeps in per cent: room for the table and
-// for pass CTAs; the rest of the SM's 256 KB is L1, where the loads in flight
-// live (with the largest carve-out the sweep at N = 262144 took 977 us).
-constexpr int kDirectCarveout = 44;
 constexpr int kBatchCarveout = 72;  // the ensemble's cluster passes need up to 74 KB a CTA
 constexpr int kFinishThreads = 256;
 constexpr int kFinishWarps = kFinishThreads / 32;

@@ -261,19 +261,6 @@ __device__ __forceinline__ void assemble_pair64(const DevFault<double>& f, int m
   *Yc = make_double2(tr + si, sr - ti);
 }
 
-// Precision-form assembly of one coefficient n of the full spectrum (the
-// four-step passes): the pair (m, N-m), m = min(n, N-n), in FP32 from the
-// FP32 per-mode inputs, Y[n] its half; U, Q of mode m are kept (pass 2) by
-// the thread with n <= N/2.
-__device__ __forceinline__ float2 assemble32_at(const DevFault<float>& f, int n, int pass, int m_dt, double dt) {
-  const int N = f.N, half = N >> 1;
-  const int m = n <= half ? n : N - n;
-  const ModeIn in = load_mode_in(f, m, m_dt, dt);
-  float2 Ym, Yc;
-  assemble_pair32(f, m, f.Z[m], f.Z[(N - m) & (N - 1)], n <= half ? pass : 0, in, &Ym, &Yc);
-  return n <= half ? Ym : Yc;
-}
-
 // Column pass: for n1 in this CTA's B columns, transform x[n1 + N1 n2] over
 // n2 (length N2), multiply by exp(-+2 pi i n1 k2 / N), store to
 // out[k2 N1 + n1].
@@ -311,25 +298,12 @@ __device__ __forceinline__ void col_body(const FftGeom& g, const Cx<R>* __restri
     if (PRO == PRO_LOAD) {
       v = in[n];
     } else if (PRO == PRO_PASS) {
-      // predictor slip rate of this pass (Sec. 3.3): V, then (V + V1)/2; the
-      // precision form has Vbar + i kappa Vbar ready in FP32 (written by the
-      // commit for pass 1, by the pass-1 Newton for pass 2)
-      if constexpr (sizeof(R) == 4) {
-        if (f.zin1) {
-          v = (pass == 1) ? f.zin1[n] : f.zin2[n];
-          buf[b * M + n2] = v;
-          continue;
-        }
-      }
+      // predictor slip rate of this pass (Sec. 3.3): V, then (V + V1)/2
       const double vb = (pass == 1) ? f.V[n] : 0.5 * (f.V[n] + f.V1[n]);
       v.x = static_cast<R>(vb);
       v.y = static_cast<R>(f.kappa[n] * vb);
     } else {
-      if constexpr (sizeof(R) == 4) {
-        v = f.U2f ? assemble32_at(f, n, pass, m_dt, dt) : assemble<R>(f, n, pass, m_dt, dt);
-      } else {
-        v = assemble<R>(f, n, pass, m_dt, dt);
-      }
+      v = assemble<R>(f, n, pass, m_dt, dt);
     }
     buf[b * M + n2] = v;
   }
@@ -1003,6 +977,333 @@ __global__ void k_row_b(const FftGeom g, const DevFault<R>* __restrict__ fs) {
   const DevFault<R>& f = fs[blockIdx.y];
   row_body<R, INV>(g, f.tw, f.zt, INV ? f.y : f.Z, INV ? R(1.0 / g.N) : R(1), f.status);
 }
+
+// ------------------------------------------- large passes (three launches)
+// The FP32 spectral pass above kFusedMaxN, on every SM: N = N1 N2 (N1 = N2 or 2 N2), both directions as
+// a column transform (length N2 over n2, index n1 + N1 n2), a twiddle
+// w_N^{n1 k2} and a row transform (length N1 over n1) to index k2 + N2 k1.
+//   k_pass_col   forward columns
+//   k_pass_mid   forward rows k2 and N2 - k2 (which hold the partners m, N - m
+//                of the assembly), the assembly in place, and the inverse
+//                columns: the modes of row k2 are those of the inverse columns
+//                n1 = k2 (and k2 + N2 when N1 = 2 N2), so nothing leaves the
+//                CTA between the two directions
+//   k_pass_row   inverse rows, scaled, to tau_el + i sigma_el
+// A thread takes three radix-2 stages at a time in registers (8 values; the
+// same butterflies and twiddles as one stage at a time, so results round the
+// same), padded so that the 64-bit accesses are free of bank conflicts.  At
+// these sizes the arrays sit in L2 and the pass is bound by its chain of
+// latencies: launches, loads, barriers.  Quasi-dynamic steps (two passes, two
+// Newton launches, commit), against four kernels a pass with a barrier pair
+// per radix-2 stage: N = 32768 45 against 72 us, 65536 53 against 88, 131072
+// 74 against 126, 262144 119 against 175 us.  Starting each kernel early behind the one
+// before it (griddepcontrol) was slower (103 us at N = 131072; the waiting
+// CTAs also keep the next step's sweep out).
+// Complex products of the passes, with the roundings spelled out: these are
+// the ones the compiler chose for the same products of one stage at a time
+// (another choice moves a quasi-dynamic shear traction of 1e-4 of the normal
+// one by 1e-4 of itself).
+__device__ __forceinline__ float2 bfly_mul(float2 a, float2 w) {
+  return make_float2(fmaf(a.x, w.x, -(a.y * w.y)), fmaf(a.y, w.x, a.x * w.y));
+}
+__device__ __forceinline__ float2 turn_mul(float2 a, float2 w) {
+  return make_float2(fmaf(a.x, w.x, -(a.y * w.y)), fmaf(a.x, w.y, a.y * w.x));
+}
+__host__ __device__ constexpr int fft_pad(int i) { return i + (i >> 3); }
+// Values of one transform of length 2^LG with padding.
+template <int LG> constexpr int kFftLen = fft_pad(1 << LG);
+
+// K radix-2 decimation-in-frequency stages (K = 1, 2, 3) of a transform of
+// length M = 2^LG, after lgs stages, for group g of the M / 2^K: values q + s
+// (p + j n / 2^K) to q + s (2^K p + j'), n = M >> lgs, s = 2^lgs.
+template <int K, int LG, bool INV, class C>
+__device__ __forceinline__ void fft_load(const C* buf, const C* twm, int lgs, int g, C (&v)[1 << K]) {
+  constexpr int M = 1 << LG, R = 1 << K;
+  const int s = 1 << lgs;
+  const int p = g >> lgs;
+  const int hop = M >> (lgs + K);  // n / 2^K
+#pragma unroll
+  for (int j = 0; j < R; ++j) v[j] = buf[fft_pad(g + j * (M / R))];  // q + s (p + j hop): s hop = M / R
+#pragma unroll
+  for (int k = 0; k < K; ++k) {
+    // branches of 2^(K - k) values; pairs half a branch apart
+    const int len = R >> k, h = len >> 1;
+#pragma unroll
+    for (int j = 0; j < R / 2; ++j) {
+      if (j < h) {
+        C w = twm[((p + j * hop) << (lgs + k)) & (M / 2 - 1)];
+        if (INV) w.y = -w.y;
+#pragma unroll
+        for (int b = 0; b < R; ++b) {
+          if (b < (1 << k)) {
+            const C a = v[b * len + j], c = v[b * len + j + h];
+            v[b * len + j] = cadd(a, c);
+            v[b * len + j + h] = bfly_mul(csub(a, c), w);
+          }
+        }
+      }
+    }
+  }
+}
+template <int K, int LG, class C>
+__device__ __forceinline__ void fft_store(C* buf, int lgs, int g, const C (&v)[1 << K]) {
+  constexpr int R = 1 << K;
+  const int s = 1 << lgs;
+  const int p = g >> lgs, q = g & (s - 1);
+#pragma unroll
+  for (int j = 0; j < R; ++j) {
+    // v[j]: stage k took the branch bit K - 1 - k of j, which adds s 2^k
+    int o = 0;
+#pragma unroll
+    for (int k = 0; k < K; ++k)
+      if (j & (1 << (K - 1 - k))) o += 1 << k;
+    buf[fft_pad(q + s * (R * p + o))] = v[j];
+  }
+}
+
+// Transforms of length 2^LG side by side in buf (kFftLen<LG> apart), one
+// group of 8 values a thread, all threads of the CTA.
+template <int LG, bool INV, class C>
+__device__ __forceinline__ void fft_fused(C* buf, const C* twm, int tid) {
+  constexpr int T = (1 << LG) / 8;
+  C* b = buf + (tid / T) * kFftLen<LG>;
+  const int g = tid % T;
+#pragma unroll
+  for (int lgs = 0; lgs + 3 <= LG; lgs += 3) {
+    C v[8];
+    fft_load<3, LG, INV>(b, twm, lgs, g, v);
+    __syncthreads();
+    fft_store<3, LG>(b, lgs, g, v);
+    __syncthreads();
+  }
+  constexpr int rest = LG % 3, lgs = LG - rest;
+  if constexpr (rest == 2) {
+    C v[2][4];
+#pragma unroll
+    for (int q = 0; q < 2; ++q) fft_load<2, LG, INV>(b, twm, lgs, g + q * T, v[q]);
+    __syncthreads();
+#pragma unroll
+    for (int q = 0; q < 2; ++q) fft_store<2, LG>(b, lgs, g + q * T, v[q]);
+    __syncthreads();
+  } else if constexpr (rest == 1) {
+    C v[4][2];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) fft_load<1, LG, INV>(b, twm, lgs, g + q * T, v[q]);
+    __syncthreads();
+#pragma unroll
+    for (int q = 0; q < 4; ++q) fft_store<1, LG>(b, lgs, g + q * T, v[q]);
+    __syncthreads();
+  }
+}
+
+// Columns (rows) per CTA of the outer kernels: four, 32 or 64 contiguous bytes
+// a segment, while that leaves 128 CTAs, else two or one.
+__host__ __device__ constexpr int pass_cols(int lines) { return lines >= 512 ? 4 : (lines >= 256 ? 2 : 1); }
+
+template <int LG1, int LG2> struct PassGeom {
+  static constexpr int N1 = 1 << LG1, N2 = 1 << LG2, N = N1 * N2;
+  static constexpr int Bc = pass_cols(N1), Br = pass_cols(N2);
+  static constexpr int tcol = Bc * N2 / 8, trow = Br * N1 / 8, tmid = 2 * N1 / 8;
+};
+
+template <int LG1, int LG2>
+__device__ __forceinline__ void pass_col_body(const DevFault<float>& f, int pass) {
+  using G = PassGeom<LG1, LG2>;
+  using C = float2;
+  constexpr int T = G::tcol, B = G::Bc, N2 = G::N2, per = B * N2 / T;
+  __shared__ __align__(16) C buf[B * kFftLen<LG2>];
+  __shared__ __align__(16) C twm[N2 / 2];
+  const int tid = threadIdx.x, c0 = blockIdx.x * B;
+  for (int j = tid; j < N2 / 2; j += T) twm[j] = f.tw[j * G::N1];
+  C w[per];
+#pragma unroll
+  for (int q = 0; q < per; ++q) {
+    const int t = tid + q * T;
+    w[q] = f.tw[(c0 + t % B) * (t / B)];  // w_N^{n1 k2} of the outputs
+  }
+  reset_newton_stats(f, pass, blockIdx.x == 0 && tid == 0);
+  if (*f.status) return;
+#pragma unroll
+  for (int q = 0; q < per; ++q) {
+    const int t = tid + q * T;
+    const int n = c0 + t % B + G::N1 * (t / B);
+    buf[(t % B) * kFftLen<LG2> + fft_pad(t / B)] = pass == 1 ? f.zin1[n] : f.zin2[n];
+  }
+  __syncthreads();
+  fft_fused<LG2, false>(buf, twm, tid);
+#pragma unroll
+  for (int q = 0; q < per; ++q) {
+    const int t = tid + q * T;
+    f.zt[(t / B) * G::N1 + c0 + t % B] = turn_mul(buf[(t % B) * kFftLen<LG2> + fft_pad(t / B)], w[q]);
+  }
+}
+
+template <int LG1, int LG2>
+__device__ __forceinline__ void pass_mid_body(const DevFault<float>& f, int pass, int m_dt, double dt) {
+  using G = PassGeom<LG1, LG2>;
+  using C = float2;
+  constexpr int T = G::tmid, N1 = G::N1, N2 = G::N2, N = G::N, half = N / 2;
+  constexpr int LR = kFftLen<LG1>, LC = kFftLen<LG2>;
+  constexpr int cols = N1 / N2;                      // inverse columns per row
+  constexpr int len = 2 * LR + (cols == 1 ? 0 : 2 * cols * LC);
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  C* buf = reinterpret_cast<C*>(smem_raw);
+  C* tw1 = buf + len;                                // length-N1 twiddles
+  C* tw2 = tw1 + N1 / 2;                             // length-N2 twiddles
+  const int tid = threadIdx.x, c = blockIdx.x;
+  const int rowA = c, rowB = c == 0 ? N2 / 2 : N2 - c;
+  for (int j = tid; j < N1 / 2; j += T) tw1[j] = f.tw[j * N2];
+  for (int j = tid; j < N2 / 2; j += T) tw2[j] = f.tw[j * N1];
+  // pairs (m, N - m) of the two rows, four a thread: element i of row A and
+  // its partner i' of row B; CTA 0 pairs within its rows (row 0: i and N1 -
+  // i, row N2 / 2: i and N1 - 1 - i), i < N1 / 2, and mode N / 2 besides
+  auto pair = [&](int q, int* ra, int* ia, int* rb, int* ib) {
+    const int i = tid + q * T;
+    if (c > 0) {
+      *ra = 0;
+      *rb = 1;
+      *ia = i;
+      *ib = N1 - 1 - i;
+    } else {
+      const int r = i / (N1 / 2), k = i % (N1 / 2);
+      *ra = *rb = r;
+      *ia = k;
+      *ib = r == 0 ? (N1 - k) & (N1 - 1) : N1 - 1 - k;
+    }
+  };
+  auto mode = [&](int r, int i) { return (r == 0 ? rowA : rowB) + N2 * i; };
+  ModeIn in[4];
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    int ra, ia, rb, ib;
+    pair(q, &ra, &ia, &rb, &ib);
+    const int m = mode(ra, ia);
+    in[q] = load_mode_in(f, m <= half ? m : N - m, m_dt, dt);
+  }
+  if (*f.status) return;
+#pragma unroll
+  for (int q = 0; q < 8; ++q) {
+    const int t = tid + q * T;
+    const int r = t / N1, i = t % N1;
+    buf[r * LR + fft_pad(i)] = f.zt[(r == 0 ? rowA : rowB) * N1 + i];
+  }
+  __syncthreads();
+  fft_fused<LG1, false>(buf, tw1, tid);
+  // in place where the rows are the inverse columns, else to the second
+  // buffer: element i of row r is value i / cols of column (r, i % cols)
+  C* const ob = cols == 1 ? buf : buf + 2 * LR;
+  auto put = [&](int r, int i, C v) { ob[(r * cols + i % cols) * LC + fft_pad(i / cols)] = v; };
+  auto one = [&](int ra, int ia, int rb, int ib, const ModeIn& mi) {
+    const int m = mode(ra, ia);
+    const bool lead = m <= half;
+    const C a = buf[ra * LR + fft_pad(ia)], b = buf[rb * LR + fft_pad(ib)];
+    C Ym, Yc;
+    assemble_pair32(f, lead ? m : N - m, lead ? a : b, lead ? b : a, pass, mi, &Ym, &Yc);
+    put(ra, ia, lead ? Ym : Yc);
+    if (rb != ra || ib != ia) put(rb, ib, lead ? Yc : Ym);
+  };
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    int ra, ia, rb, ib;
+    pair(q, &ra, &ia, &rb, &ib);
+    one(ra, ia, rb, ib, in[q]);
+  }
+  // mode N / 2: element N1 / 2 of row 0, its own partner
+  if (c == 0 && tid == 0) one(0, N1 / 2, 0, N1 / 2, load_mode_in(f, half, m_dt, dt));
+  __syncthreads();
+  fft_fused<LG2, true>(ob, tw2, tid);
+#pragma unroll
+  for (int q = 0; q < 8; ++q) {
+    const int t = tid + q * T;
+    const int k2 = t % N2, col = t / N2;
+    const int n1 = (col / cols == 0 ? rowA : rowB) + N2 * (col % cols);
+    C w = f.tw[n1 * k2];
+    w.y = -w.y;
+    f.Z[k2 * N1 + n1] = turn_mul(ob[col * LC + fft_pad(k2)], w);
+  }
+}
+
+template <int LG1, int LG2>
+__device__ __forceinline__ void pass_row_body(const DevFault<float>& f) {
+  using G = PassGeom<LG1, LG2>;
+  using C = float2;
+  constexpr int T = G::trow, B = G::Br, N1 = G::N1, per = B * N1 / T;
+  __shared__ __align__(16) C buf[B * kFftLen<LG1>];
+  __shared__ __align__(16) C twm[N1 / 2];
+  const int tid = threadIdx.x, c0 = blockIdx.x * B;
+  for (int j = tid; j < N1 / 2; j += T) twm[j] = f.tw[j * G::N2];
+  if (*f.status) return;
+#pragma unroll
+  for (int q = 0; q < per; ++q) {
+    const int t = tid + q * T;
+    buf[(t / N1) * kFftLen<LG1> + fft_pad(t % N1)] = f.Z[(c0 + t / N1) * N1 + t % N1];
+  }
+  __syncthreads();
+  fft_fused<LG1, true>(buf, twm, tid);
+  constexpr float scale = 1.0f / G::N;
+#pragma unroll
+  for (int q = 0; q < per; ++q) {
+    const int t = tid + q * T;
+    C v = buf[(t % B) * kFftLen<LG1> + fft_pad(t / B)];
+    v.x *= scale;
+    v.y *= scale;
+    f.y[c0 + t % B + G::N2 * (t / B)] = v;
+  }
+}
+
+template <int LG1, int LG2>
+__global__ void __launch_bounds__(PassGeom<LG1, LG2>::tcol)
+    k_pass_col(const __grid_constant__ DevFault<float> f, int pass) {
+  pass_col_body<LG1, LG2>(f, pass);
+}
+template <int LG1, int LG2>
+__global__ void __launch_bounds__(PassGeom<LG1, LG2>::tmid)
+    k_pass_mid(const __grid_constant__ DevFault<float> f, int pass, int m_dt, double dt) {
+  pass_mid_body<LG1, LG2>(f, pass, m_dt, dt);
+}
+template <int LG1, int LG2>
+__global__ void __launch_bounds__(PassGeom<LG1, LG2>::trow) k_pass_row(const __grid_constant__ DevFault<float> f) {
+  pass_row_body<LG1, LG2>(f);
+}
+// Ensembles: member blockIdx.y.
+template <int LG1, int LG2>
+__global__ void __launch_bounds__(PassGeom<LG1, LG2>::tcol) k_pass_col_b(const DevFault<float>* __restrict__ fs, int pass) {
+  pass_col_body<LG1, LG2>(fs[blockIdx.y], pass);
+}
+template <int LG1, int LG2>
+__global__ void __launch_bounds__(PassGeom<LG1, LG2>::tmid)
+    k_pass_mid_b(const DevFault<float>* __restrict__ fs, int pass, int m_dt) {
+  const DevFault<float>& f = fs[blockIdx.y];
+  pass_mid_body<LG1, LG2>(f, pass, m_dt, m_dt * f.dt_min);
+}
+template <int LG1, int LG2>
+__global__ void __launch_bounds__(PassGeom<LG1, LG2>::trow) k_pass_row_b(const DevFault<float>* __restrict__ fs) {
+  pass_row_body<LG1, LG2>(fs[blockIdx.y]);
+}
+
+template <int LG1, int LG2>
+static constexpr size_t pass_mid_smem() {
+  constexpr int cols = (1 << LG1) >> LG2;
+  return static_cast<size_t>(2 * kFftLen<LG1> + (cols == 1 ? 0 : 2 * cols * kFftLen<LG2>) + (1 << LG1) / 2 +
+                             (1 << LG2) / 2) * sizeof(float2);
+}
+
+// fn(lg N1, lg N2) as integral constants for the sizes of the three-launch
+// pass.
+template <class F>
+static void with_pass(int N, F&& fn) {
+  using std::integral_constant;
+  switch (31 - __builtin_clz(static_cast<unsigned>(N))) {
+    case 15: fn(integral_constant<int, 8>{}, integral_constant<int, 7>{}); break;
+    case 16: fn(integral_constant<int, 8>{}, integral_constant<int, 8>{}); break;
+    case 17: fn(integral_constant<int, 9>{}, integral_constant<int, 8>{}); break;
+    case 18: fn(integral_constant<int, 9>{}, integral_constant<int, 9>{}); break;
+    case 19: fn(integral_constant<int, 10>{}, integral_constant<int, 9>{}); break;
+    case 20: fn(integral_constant<int, 10>{}, integral_constant<int, 10>{}); break;
+    default: break;
+  }
+}
+static_assert(kFusedMaxN == 1 << 14, "with_pass covers the sizes above");
 
 // ---------------------------------------------------- history convolution
 // Ring slot i of mode n (i = 0 newest) holds the spectra of the interval
@@ -2650,23 +2951,33 @@ void launch_spectral(const DevFault<R>& f, int pass, int m_dt, cudaStream_t st, 
         constexpr int LG = decltype(lg)::value;
         if constexpr ((1 << LG) <= kCluster64MaxN) {
           constexpr int C = cluster64_ctas(1 << LG);
-          launch_attr(k_spectral_cluster64<LG>, dim3(C), dim3(cluster64_threads(f.N)), cluster64_smem(f.N), st, C, pass == 2,
-                      started, f, pass, m_dt, dt);
+          launch_attr(k_spectral_cluster64<LG>, dim3(C), dim3(cluster64_threads(f.N)), cluster64_smem(f.N), st, C,
+                      pass == 2, started, f, pass, m_dt, dt);
         }
       });
       return;
     }
   }
-  const size_t cs = col_smem<R>(g), rs = row_smem<R>(g);
-  auto kfa = k_col<R, false, PRO_PASS>;
-  auto kfb = k_row<R, false>;
-  auto kia = k_col<R, true, PRO_ASSEMBLE>;
-  auto kib = k_row<R, true>;
-  launch_attr(kfa, dim3(g.N1 / g.Bc), dim3(g.tc), cs, st, 1, false, started, g, static_cast<const Cx<R>*>(f.tw),
-              static_cast<const Cx<R>*>(nullptr), f.zt, f, pass, m_dt, dt);
-  kfb<<<g.N2 / g.Br, g.tr, rs, st>>>(g, f.tw, f.zt, f.Z, R(1), f.status);
-  kia<<<g.N1 / g.Bc, g.tc, cs, st>>>(g, f.tw, nullptr, f.zt, f, pass, m_dt, dt);
-  kib<<<g.N2 / g.Br, g.tr, rs, st>>>(g, f.tw, f.zt, f.y, R(1.0 / g.N), f.status);
+  if constexpr (sizeof(R) == 4) {
+    with_pass(f.N, [&](auto l1, auto l2) {
+      constexpr int L1 = decltype(l1)::value, L2 = decltype(l2)::value;
+      using G = PassGeom<L1, L2>;
+      launch_attr(k_pass_col<L1, L2>, dim3(G::N1 / G::Bc), dim3(G::tcol), 0, st, 1, false, started, f, pass);
+      k_pass_mid<L1, L2><<<G::N2 / 2, G::tmid, pass_mid_smem<L1, L2>(), st>>>(f, pass, m_dt, dt);
+      k_pass_row<L1, L2><<<G::N2 / G::Br, G::trow, 0, st>>>(f);
+    });
+  } else {
+    const size_t cs = col_smem<R>(g), rs = row_smem<R>(g);
+    auto kfa = k_col<R, false, PRO_PASS>;
+    auto kfb = k_row<R, false>;
+    auto kia = k_col<R, true, PRO_ASSEMBLE>;
+    auto kib = k_row<R, true>;
+    launch_attr(kfa, dim3(g.N1 / g.Bc), dim3(g.tc), cs, st, 1, false, started, g, static_cast<const Cx<R>*>(f.tw),
+                static_cast<const Cx<R>*>(nullptr), f.zt, f, pass, m_dt, dt);
+    kfb<<<g.N2 / g.Br, g.tr, rs, st>>>(g, f.tw, f.zt, f.Z, R(1), f.status);
+    kia<<<g.N1 / g.Bc, g.tc, cs, st>>>(g, f.tw, nullptr, f.zt, f, pass, m_dt, dt);
+    kib<<<g.N2 / g.Br, g.tr, rs, st>>>(g, f.tw, f.zt, f.y, R(1.0 / g.N), f.status);
+  }
 }
 
 // The Newton part of a pass (state predictor and friction solve, Sec. 3.3), started early behind the spectral part.
@@ -2895,20 +3206,30 @@ void launch_pass_batch(const FftGeom& g, const DevFault<R>* fs, int members, int
         constexpr int LG = decltype(lg)::value;
         if constexpr ((1 << LG) <= kCluster64MaxN) {
           constexpr int C = cluster64_ctas(1 << LG);
-          launch_attr(k_spectral_cluster64_b<LG>, dim3(C * members), dim3(cluster64_threads(N)), cluster64_smem(N), st, C,
-                      false, static_cast<cudaEvent_t>(nullptr), fs, pass, m_dt);
+          launch_attr(k_spectral_cluster64_b<LG>, dim3(C * members), dim3(cluster64_threads(N)), cluster64_smem(N), st,
+                      C, false, static_cast<cudaEvent_t>(nullptr), fs, pass, m_dt);
         }
       });
       k_newton_b<R><<<dim3((N + 31) / 32, members), 32, 0, st>>>(fs, pass, m_dt);
       return;
     }
   }
-  const size_t cs = col_smem<R>(g), rs = row_smem<R>(g);
-  const dim3 gc(g.N1 / g.Bc, members), gr(g.N2 / g.Br, members);
-  k_col_b<R, false, PRO_PASS><<<gc, g.tc, cs, st>>>(g, fs, pass, m_dt);
-  k_row_b<R, false><<<gr, g.tr, rs, st>>>(g, fs);
-  k_col_b<R, true, PRO_ASSEMBLE><<<gc, g.tc, cs, st>>>(g, fs, pass, m_dt);
-  k_row_b<R, true><<<gr, g.tr, rs, st>>>(g, fs);
+  if constexpr (sizeof(R) == 4) {
+    with_pass(N, [&](auto l1, auto l2) {
+      constexpr int L1 = decltype(l1)::value, L2 = decltype(l2)::value;
+      using G = PassGeom<L1, L2>;
+      k_pass_col_b<L1, L2><<<dim3(G::N1 / G::Bc, members), G::tcol, 0, st>>>(fs, pass);
+      k_pass_mid_b<L1, L2><<<dim3(G::N2 / 2, members), G::tmid, pass_mid_smem<L1, L2>(), st>>>(fs, pass, m_dt);
+      k_pass_row_b<L1, L2><<<dim3(G::N2 / G::Br, members), G::trow, 0, st>>>(fs);
+    });
+  } else {
+    const size_t cs = col_smem<R>(g), rs = row_smem<R>(g);
+    const dim3 gc(g.N1 / g.Bc, members), gr(g.N2 / g.Br, members);
+    k_col_b<R, false, PRO_PASS><<<gc, g.tc, cs, st>>>(g, fs, pass, m_dt);
+    k_row_b<R, false><<<gr, g.tr, rs, st>>>(g, fs);
+    k_col_b<R, true, PRO_ASSEMBLE><<<gc, g.tc, cs, st>>>(g, fs, pass, m_dt);
+    k_row_b<R, true><<<gr, g.tr, rs, st>>>(g, fs);
+  }
   k_newton_b<R><<<dim3((N + 31) / 32, members), 32, 0, st>>>(fs, pass, m_dt);  // members use 32 per warp
 }
 
@@ -2942,10 +3263,17 @@ void configure_batch_kernels(const FftGeom& g) {
         }
       });
   }
+  if constexpr (sizeof(R) == 4) {
+  with_pass(g.N, [&](auto l1, auto l2) {
+    constexpr int L1 = decltype(l1)::value, L2 = decltype(l2)::value;
+    allow_smem(k_pass_mid_b<L1, L2>, pass_mid_smem<L1, L2>());
+  });
+  } else {
   allow_smem(k_col_b<R, false, PRO_PASS>, col_smem<R>(g));
   allow_smem(k_col_b<R, true, PRO_ASSEMBLE>, col_smem<R>(g));
   allow_smem(k_row_b<R, false>, row_smem<R>(g));
   allow_smem(k_row_b<R, true>, row_smem<R>(g));
+  }
 }
 
 template <class R>
@@ -3128,11 +3456,21 @@ void configure_kernels(const FftGeom& g) {
         }
       });
   }
+  if constexpr (sizeof(R) == 4) {
+  with_pass(g.N, [&](auto l1, auto l2) {
+    constexpr int L1 = decltype(l1)::value, L2 = decltype(l2)::value;
+    allow_smem(k_pass_mid<L1, L2>, pass_mid_smem<L1, L2>());
+    cudaFuncSetAttribute(k_pass_col<L1, L2>, cudaFuncAttributePreferredSharedMemoryCarveout, kDirectCarveout);
+    cudaFuncSetAttribute(k_pass_mid<L1, L2>, cudaFuncAttributePreferredSharedMemoryCarveout, kDirectCarveout);
+    cudaFuncSetAttribute(k_pass_row<L1, L2>, cudaFuncAttributePreferredSharedMemoryCarveout, kDirectCarveout);
+  });
+  } else {
   const size_t cs = col_smem<R>(g), rs = row_smem<R>(g);
   allow_smem(k_col<R, false, PRO_PASS>, cs);
   allow_smem(k_col<R, true, PRO_ASSEMBLE>, cs);
   allow_smem(k_row<R, false>, rs);
   allow_smem(k_row<R, true>, rs);
+  }
   const FftGeom g64 = make_geom(g.N, sizeof(double2));
   allow_smem(k_col<double, false, PRO_LOAD>, col_smem<double>(g64));
   allow_smem(k_col<double, true, PRO_LOAD>, col_smem<double>(g64));

@@ -184,6 +184,14 @@ struct SweepBarrier {
   long long limit;
   int members;
 };
+// Shared memory carve-out of the direct sweep in per cent: room for its table
+// and for pass CTAs; the rest of the SM's 256 KB is L1, where the loads in
+// flight live (with the largest carve-out the sweep at N = 262144 took 977 us
+// instead of 783).  A kernel for which the driver would choose another one
+// waits until the SM is idle, so the passes that run beside the sweep ask for
+// the same (left to the driver, the passes at N = 65536 began only when the
+// sweep had ended).
+constexpr int kDirectCarveout = 44;
 template <class R> void configure_direct();
 // Resident CTAs per SM of the direct sweep (gen: with a weight table of
 // `pieces` pieces).
