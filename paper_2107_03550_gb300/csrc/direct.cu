@@ -511,7 +511,10 @@ int direct_blocks_per_sm(bool gen, int P, bool persist) {
 template <class R>
 void launch_direct(const DirectTable<R>& t, const DevFault<R>& f, int m, int grid, bool ahead, cudaStream_t st,
                    cudaEvent_t swept) {
-  if (t.nitems == 0) return;
+  if (t.nitems == 0) {
+    if (swept) cudaEventRecord(swept, st);  // no history (the quasi-dynamic limit)
+    return;
+  }
   double2* oT = ahead ? f.BT : f.AT;
   double2* oN = ahead ? f.BN : f.AN;
   float2* fT = ahead ? nullptr : f.AT32;

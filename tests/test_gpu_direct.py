@@ -34,3 +34,21 @@ def test_direct_sums_match_the_bulk_async_form(N, precision, kw, tol):
         for a, b in zip(direct, bulk):
             assert rel(a, b) <= tol, (m, rel(a, b))
     g.close()
+
+
+def test_sweep_mark_without_history():
+    # the quasi-dynamic limit has nothing to sweep: the mark between sweep and
+    # finish is recorded all the same
+    import torch
+    g = gpu_for(seamount_rupture(N=256), eta_w=0.0)
+    st = torch.cuda.current_stream()
+    g.set_stream(st)
+    a, b, c = (torch.cuda.Event(enable_timing=True) for _ in range(3))
+    b.record()
+    torch.cuda.synchronize()
+    a.record()
+    g.history_enqueue(1, sweep_done=b)
+    c.record()
+    torch.cuda.synchronize()
+    assert a.elapsed_time(b) >= 0.0 and b.elapsed_time(c) >= 0.0
+    g.close()
