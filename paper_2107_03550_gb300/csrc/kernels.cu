@@ -286,8 +286,9 @@ __device__ __forceinline__ void col_body(const FftGeom& g, const Cx<R>* __restri
   C* twm = buf + B * M;
   const int tid = threadIdx.x, nth = blockDim.x;
   if (PRO != PRO_LOAD) reset_newton_stats(f, pass, blockIdx.x == 0 && tid == 0);
-  // the status word only changes in k_newton, never while this kernel runs
-  if (PRO != PRO_LOAD && *f.status) return;
+  // one decision per CTA: a Newton kernel of the adaptive run's other branch
+  // may set the status word while this kernel runs
+  if (PRO != PRO_LOAD && __syncthreads_or(*f.status != 0u)) return;
   for (int j = tid; j < (M >> 1); j += nth) twm[j] = tw[j * g.N1];
   const int c0 = blockIdx.x * B;
   for (int t = tid; t < B * M; t += nth) {
@@ -946,7 +947,7 @@ __device__ __forceinline__ void row_body(const FftGeom& g, const Cx<R>* __restri
   const int M = g.N1, B = g.Br;
   C* twm = buf + B * M;
   const int tid = threadIdx.x, nth = blockDim.x;
-  if (status && *status) return;
+  if (status && __syncthreads_or(*status != 0u)) return;  // one decision per CTA, as in col_body
   for (int j = tid; j < (M >> 1); j += nth) twm[j] = tw[j * g.N2];
   const int c0 = blockIdx.x * B;
   for (int t = tid; t < B * M; t += nth) {
@@ -1122,14 +1123,16 @@ __device__ __forceinline__ void pass_col_body(const DevFault<float>& f, int pass
     w[q] = f.tw[(c0 + t % B) * (t / B)];  // w_N^{n1 k2} of the outputs
   }
   reset_newton_stats(f, pass, blockIdx.x == 0 && tid == 0);
-  if (*f.status) return;
+  const unsigned failed = *f.status;
 #pragma unroll
   for (int q = 0; q < per; ++q) {
     const int t = tid + q * T;
     const int n = c0 + t % B + G::N1 * (t / B);
     buf[(t % B) * kFftLen<LG2> + fft_pad(t / B)] = pass == 1 ? f.zin1[n] : f.zin2[n];
   }
-  __syncthreads();
+  // one decision per CTA: a Newton kernel of the adaptive run's other branch
+  // may set the status word while this kernel runs
+  if (__syncthreads_or(failed != 0u)) return;
   fft_fused<LG2, false>(buf, twm, tid);
 #pragma unroll
   for (int q = 0; q < per; ++q) {
@@ -1180,14 +1183,14 @@ __device__ __forceinline__ void pass_mid_body(const DevFault<float>& f, int pass
     const int m = mode(ra, ia);
     in[q] = load_mode_in(f, m <= half ? m : N - m, m_dt, dt);
   }
-  if (*f.status) return;
+  const unsigned failed = *f.status;
 #pragma unroll
   for (int q = 0; q < 8; ++q) {
     const int t = tid + q * T;
     const int r = t / N1, i = t % N1;
     buf[r * LR + fft_pad(i)] = f.zt[(r == 0 ? rowA : rowB) * N1 + i];
   }
-  __syncthreads();
+  if (__syncthreads_or(failed != 0u)) return;  // one decision per CTA, as in pass_col_body
   fft_fused<LG1, false>(buf, tw1, tid);
   // in place where the rows are the inverse columns, else to the second
   // buffer: element i of row r is value i / cols of column (r, i % cols)
@@ -1232,13 +1235,13 @@ __device__ __forceinline__ void pass_row_body(const DevFault<float>& f) {
   __shared__ __align__(16) C twm[N1 / 2];
   const int tid = threadIdx.x, c0 = blockIdx.x * B;
   for (int j = tid; j < N1 / 2; j += T) twm[j] = f.tw[j * G::N2];
-  if (*f.status) return;
+  const unsigned failed = *f.status;
 #pragma unroll
   for (int q = 0; q < per; ++q) {
     const int t = tid + q * T;
     buf[(t / N1) * kFftLen<LG1> + fft_pad(t % N1)] = f.Z[(c0 + t / N1) * N1 + t % N1];
   }
-  __syncthreads();
+  if (__syncthreads_or(failed != 0u)) return;  // one decision per CTA, as in pass_col_body
   fft_fused<LG1, true>(buf, twm, tid);
   constexpr float scale = 1.0f / G::N;
 #pragma unroll
