@@ -93,7 +93,10 @@ typedef struct sbiem_params {
                            1 the FP32 sweep streams its weights           */
   double  newton_tol;   /* |delta ln V| convergence tolerance, default 1e-12   */
   double  f0, V0;       /* reference friction and slip rate (Eq. momentum)     */
-  sbiem_alloc_fn alloc_fn; /* optional device allocator (NULL: cudaMalloc)     */
+  sbiem_alloc_fn alloc_fn; /* optional device allocator (NULL: cudaMalloc).
+                              From the first pointer that is not 64-byte
+                              aligned (freed at once) every request is 63
+                              bytes larger, to align in                      */
   sbiem_free_fn  free_fn;  /* matching free (NULL: cudaFree)                   */
   void*   alloc_user;      /* passed to alloc_fn / free_fn                     */
 } sbiem_params;

@@ -3,6 +3,7 @@
 
 #include <algorithm>
 #include <cmath>
+#include <cstdint>
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
@@ -66,6 +67,7 @@ struct sbiem_s {
   int64_t total_slots = 0, total_w = 0;
   std::vector<Chunk> chunks;
   std::vector<void*> allocs;
+  size_t alloc_pad = 0;  // asked for beyond each array (a caller's allocator of less alignment)
   int64_t device_bytes = 0;
   DevFault<double> f64{};
   DevFault<float> f32{};
@@ -150,20 +152,31 @@ struct sbiem_s {
 
 namespace {
 
+// Alignment of every device array: the widest record (DirectItem) is 64 bytes,
+// and a history slot of the FP64 form is read by one 32-byte load.  A caller's
+// allocator that once returns less is asked for that much more from then on.
+constexpr size_t kDevAlign = 64;
+
 void* dev_alloc(sbiem_s* s, size_t bytes) {
   if (bytes == 0) bytes = 16;
   void* ptr = nullptr;
   if (s->p.alloc_fn) {
-    ptr = s->p.alloc_fn(bytes, s->p.alloc_user);
+    ptr = s->p.alloc_fn(bytes + s->alloc_pad, s->p.alloc_user);
+    if (s->alloc_pad == 0 && reinterpret_cast<uintptr_t>(ptr) % kDevAlign != 0) {
+      s->alloc_pad = kDevAlign - 1;
+      if (s->p.free_fn) s->p.free_fn(ptr, s->p.alloc_user);
+      else cudaFree(ptr);
+      ptr = s->p.alloc_fn(bytes + s->alloc_pad, s->p.alloc_user);
+    }
+    bytes += s->alloc_pad;
   } else if (cudaMalloc(&ptr, bytes) != cudaSuccess) {
     ptr = nullptr;
   }
-  if (ptr) {
-    s->allocs.push_back(ptr);
-    s->device_bytes += static_cast<int64_t>(bytes);
-    cudaMemsetAsync(ptr, 0, bytes, s->stream);
-  }
-  return ptr;
+  if (!ptr) return nullptr;
+  s->allocs.push_back(ptr);  // as allocated, for the free
+  s->device_bytes += static_cast<int64_t>(bytes);
+  cudaMemsetAsync(ptr, 0, bytes, s->stream);
+  return reinterpret_cast<void*>((reinterpret_cast<uintptr_t>(ptr) + kDevAlign - 1) / kDevAlign * kDevAlign);
 }
 
 template <class T>
