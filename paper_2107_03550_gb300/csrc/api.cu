@@ -170,6 +170,7 @@ void* dev_alloc(sbiem_s* s, size_t bytes) {
     }
     bytes += s->alloc_pad;
   } else if (cudaMalloc(&ptr, bytes) != cudaSuccess) {
+    cudaGetLastError();  // reported by the caller; later calls go on
     ptr = nullptr;
   }
   if (!ptr) return nullptr;
@@ -206,6 +207,15 @@ void drop_host_graph(sbiem_s* s) {
   s->host_graph.m = 0;
 }
 
+// Frees the device arrays allocated after the first `mark` (nothing uses them).
+void free_since(sbiem_s* s, size_t mark) {
+  for (size_t k = mark; k < s->allocs.size(); ++k) {
+    if (s->p.free_fn) s->p.free_fn(s->allocs[k], s->p.alloc_user);
+    else cudaFree(s->allocs[k]);
+  }
+  s->allocs.resize(mark);
+}
+
 void free_all(sbiem_s* s) {
   drop_host_graph(s);
   for (auto& kv : s->graphs) cudaGraphExecDestroy(kv.second);
@@ -221,11 +231,7 @@ void free_all(sbiem_s* s) {
   for (auto& e : s->pev)
     if (e) cudaEventDestroy(e);
   s->pev.clear();
-  for (void* ptr : s->allocs) {
-    if (s->p.free_fn) s->p.free_fn(ptr, s->p.alloc_user);
-    else cudaFree(ptr);
-  }
-  s->allocs.clear();
+  free_since(s, 0);
   if (s->h_out) cudaFreeHost(s->h_out);
   if (s->h_status) cudaFreeHost(s->h_status);
   if (s->h_steps) cudaFreeHost(s->h_steps);
@@ -512,16 +518,32 @@ void ring_undo(sbiem_s* s, int m, int dir, cudaStream_t st) {
   else launch_ring_undo<double>(s->f64, m, s->undo, dir, st);
 }
 
+// Buffers allocated on first use, all of them or none: where `get` fails, what
+// it allocated is given back, so that a later call can try again.
+template <class F>
+bool all_or_none(sbiem_s* s, F&& get) {
+  const size_t mark = s->allocs.size();
+  const int64_t bytes = s->device_bytes;
+  if (get()) return true;
+  cudaStreamSynchronize(s->stream);  // the new arrays are being zeroed
+  free_since(s, mark);
+  s->device_bytes = bytes;
+  return false;
+}
+
 // Device buffers of the state snapshot (allocated on first use).
 bool ensure_snapshot(sbiem_s* s) {
-  bool ok = true;
-  if (!s->snap) {
-    s->snap = alloc_n<double>(s, static_cast<size_t>(6) * s->N + 1, &ok);
-    s->snap_spec = alloc_n<double2>(s, static_cast<size_t>(2) * s->nmodes, &ok);
-    s->snap_head = alloc_n<int32_t>(s, s->nmodes, &ok);
-    s->snap_steps = alloc_n<long long>(s, 1, &ok);
-  }
-  return ok && s->snap && s->snap_spec && s->snap_head && s->snap_steps;
+  if (s->snap) return true;
+  const bool ok = all_or_none(s, [&] {
+    bool got = true;
+    s->snap = alloc_n<double>(s, static_cast<size_t>(6) * s->N + 1, &got);
+    s->snap_spec = alloc_n<double2>(s, static_cast<size_t>(2) * s->nmodes, &got);
+    s->snap_head = alloc_n<int32_t>(s, s->nmodes, &got);
+    s->snap_steps = alloc_n<long long>(s, 1, &got);
+    return got;
+  });
+  if (!ok) s->snap = nullptr;
+  return ok;
 }
 
 // Save (save = true) or restore the committed state that a step changes.
@@ -554,6 +576,28 @@ bool trial_buffers(sbiem_s* s, const DevFault<R>& f, DevFault<R>& t) {
   }
   t.it_sum = alloc_n<unsigned long long>(s, 1, &ok);
   t.it_max = alloc_n<int>(s, 1, &ok);
+  return ok;
+}
+
+// What the adaptive run keeps besides the snapshot (allocated at its first call).
+bool ensure_run(sbiem_s* s) {
+  if (s->undo) return true;
+  for (cudaEvent_t* e : {&s->ev_sums, &s->ev_trial})
+    if (!*e && cudaEventCreateWithFlags(e, cudaEventDisableTiming) != cudaSuccess) return false;
+  if (!s->h_trial && cudaMallocHost(&s->h_trial, sizeof(TrialReport)) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  const bool ok = all_or_none(s, [&] {
+    bool got = true;
+    s->dfull = alloc_n<double>(s, s->N, &got);
+    s->trial_work = alloc_n<unsigned long long>(s, 2, &got);
+    got = got && (s->fp32() ? trial_buffers<float>(s, s->f32, s->trial32) : trial_buffers<double>(s, s->f64, s->trial64));
+    const size_t slot = s->fp32() ? sizeof(Slot32) : sizeof(Slot64);
+    if (got) s->undo = dev_alloc(s, slot * static_cast<size_t>(std::max<int64_t>(s->total_slots, 1)));
+    return got && s->undo;
+  });
+  if (!ok) s->undo = nullptr;
   return ok;
 }
 
@@ -1241,19 +1285,8 @@ int sbiem_run(sbiem_t s, double t_end, double eps0, int64_t m0, int64_t m_max, i
   if (!s || !(eps0 > 0) || m0 < 1 || m_max < 1 || max_steps < 0) return fail(SBIEM_ERR_INVALID, "bad argument");
   s->lag_m = -1;  // trial steps and rollbacks below compute their own sums
   auto& f = s->f64;
-  bool ok = ensure_snapshot(s);
-  if (!s->undo) {
-    s->dfull = alloc_n<double>(s, s->N, &ok);
-    s->trial_work = alloc_n<unsigned long long>(s, 2, &ok);
-    ok = ok && (s->fp32() ? trial_buffers<float>(s, s->f32, s->trial32) : trial_buffers<double>(s, f, s->trial64));
-    for (cudaEvent_t* e : {&s->ev_sums, &s->ev_trial})
-      if (ok && !*e) ok = cudaEventCreateWithFlags(e, cudaEventDisableTiming) == cudaSuccess;
-    if (ok && !s->h_trial) ok = cudaMallocHost(&s->h_trial, sizeof(TrialReport)) == cudaSuccess;
-    const size_t slot = s->fp32() ? sizeof(Slot32) : sizeof(Slot64);
-    if (ok) s->undo = dev_alloc(s, slot * static_cast<size_t>(std::max<int64_t>(s->total_slots, 1)));
-    if (!s->undo) ok = false;
-  }
-  if (!ok) return fail(SBIEM_ERR_NOMEM, "adaptive run: snapshot allocation failed");
+  if (!ensure_snapshot(s) || !ensure_run(s))
+    return fail(SBIEM_ERR_NOMEM, "adaptive run: snapshot allocation failed");
   // m: a power of two in [1, 2^30]
   auto pow2_floor = [](int64_t v) {
     int64_t p = 1;
