@@ -267,8 +267,9 @@ int sbiem_load(sbiem_t* out, const char* path, const sbiem_params* alloc);
  * nodes inside the step graph as well): at the start of the step, before and
  * after the history convolution kernel, and at the end of the step.  Step k
  * (counted from the call) uses event slot k mod nslots, so nslots steps can
- * be enqueued back to back and read afterwards.  nslots = 0 disables the
- * probe.  sbiem_probe_read synchronizes on the slot's last event and returns
+ * be enqueued back to back and read afterwards.  sbiem_run marks each step of
+ * dt_min and the second half step of each attempt, all in the slot of the
+ * step before it.  nslots = 0 disables the probe.  sbiem_probe_read synchronizes on the slot's last event and returns
  * the elapsed milliseconds of that step and of its history convolution.
  * Enabling or disabling rebuilds the step graph.
  */

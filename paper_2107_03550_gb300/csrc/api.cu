@@ -466,7 +466,13 @@ int setup_device(sbiem_s* s, DevFault<R>& f, const DevFault<double>& base) {
 }
 
 void probe_mark(sbiem_s* s, int k, cudaStream_t st) {
-  if (s->pslots) cudaEventRecordWithFlags(s->pev[4 * s->pcur + k], st, cudaEventRecordExternal);
+  if (!s->pslots) return;
+  // a node of its own in a captured step (which may not record in any other
+  // way); outside a capture that flag is an error
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  cudaStreamIsCapturing(st, &cap);
+  cudaEventRecordWithFlags(s->pev[4 * s->pcur + k], st,
+                           cap == cudaStreamCaptureStatusNone ? cudaEventRecordDefault : cudaEventRecordExternal);
 }
 
 template <class R>
@@ -612,6 +618,8 @@ bool ensure_run(sbiem_s* s) {
 // grouping); the FP32 form sweeps them anew, so that the sums round as those
 // of single steps do (at the start of a rupture the static and history terms
 // nearly cancel, and a regrouped FP32 sum moved the normal traction by 1e-4).
+// With the timing probe on, the second half step, which has the GPU to itself,
+// is the one that is marked; it then sweeps in FP64 too.
 template <class R>
 int enqueue_attempt(sbiem_s* s, const DevFault<R>& f, const DevFault<R>& staging, int m) {
   const cudaStream_t st = s->stream, sd = s->side;
@@ -641,14 +649,18 @@ int enqueue_attempt(sbiem_s* s, const DevFault<R>& f, const DevFault<R>& staging
   launch_pass<R>(f, 2, h, st);
   // the whole step has read the committed state, which is saved
   CK(cudaStreamWaitEvent(st, s->ev_trial, 0));
-  constexpr bool lag = sizeof(R) == 8;
+  const bool lag = sizeof(R) == 8 && s->pslots == 0;
   if (h > 1) launch_push_multi<R>(f, h, st);
   launch_commit<R>(f, h, st, lag ? p : -1);
+  probe_mark(s, 0, st);
+  probe_mark(s, 1, st);
   if (!lag) launch_history<R>(f, h, s->hist_grid, st);
+  probe_mark(s, 2, st);
   launch_pass<R>(f, 1, h, st);
   launch_pass<R>(f, 2, h, st);
   if (h > 1) launch_push_multi<R>(f, h, st);
   launch_commit<R>(f, h, st);
+  probe_mark(s, 3, st);
   launch_trial_report(f.delta, s->dfull, s->N, f.status, s->trial_work, s->h_trial, st);
   CK(cudaGetLastError());
   return SBIEM_OK;
