@@ -27,7 +27,7 @@ namespace {
 thread_local std::string g_last_error;
 
 // Sweep shape of a new handle (chunk length x stages in flight; the direct
-// sweep where direct_form says so).
+// sweep where direct_rule says so).
 constexpr int kDefaultSweepShape = 3;
 // Largest on-chip weight table (bytes): it is read through L1 beside the
 // sweep's stages in shared memory.
@@ -278,22 +278,26 @@ void windows(const sbiem_params& p, double L, double dt_min, std::vector<int64_t
   for (size_t n = 0; n < MT.size(); ++n) M[n] = std::max(MT[n], MN[n]);
 }
 
-// Whether a handle's sweep of this shape is the direct sweep (the rule and its
-// figures stand at use_direct in kernels.cu).
-bool direct_form(const sbiem_s* s, int shape) { return shape == 3 && (!s->fp32() || s->N > kFusedMaxN); }
+// Whether a handle's sweeps of a shape are direct in some weight form at the
+// default wait limit (its tables are then set up).
+bool can_direct(const sbiem_s* s, int shape) {
+  return direct_rule(s->fp32(), s->N, shape, SBIEM_WAIT_LIMIT_DEFAULT, false, false);
+}
 
-// Whether the direct sweep takes its weights from the table (FP32, on-chip
-// weights asked for and a table there).
-bool direct_gen(const sbiem_s* s, float gen_ds_max) {
-  return s->fp32() && gen_ds_max > 0.0f && s->direct_wtab != nullptr;
+// Whether modes evaluate weights on chip (FP32, asked for and a table there).
+bool on_chip(const sbiem_s* s, float gen_ds_max) { return s->fp32() && s->f32.wtab && gen_ds_max > 0.0f; }
+
+// Whether the handle's sweep of this shape and weight form is the direct one.
+bool direct_form(const sbiem_s* s, int shape, float gen_ds_max) {
+  return direct_rule(s->fp32(), s->N, shape, s->spin_limit, on_chip(s, gen_ds_max), s->direct_wtab != nullptr);
 }
 
 // Resident CTAs per SM of a sweep shape in the weight form of gen_ds_max.
 int sweep_blocks(const sbiem_s* s, int shape, float gen_ds_max) {
-  const bool gen = s->fp32() && s->f32.wtab && gen_ds_max > 0.0f;
+  const bool gen = on_chip(s, gen_ds_max);
   int n;
-  if (direct_form(s, shape)) {
-    n = s->fp32() ? direct_blocks_per_sm<float>(direct_gen(s, gen_ds_max), s->direct_pieces, false)
+  if (direct_form(s, shape, gen_ds_max)) {
+    n = s->fp32() ? direct_blocks_per_sm<float>(gen, s->direct_pieces, false)
                   : direct_blocks_per_sm<double>(false, 0, false);
   } else {
     n = s->fp32() ? sweep_blocks_per_sm<float>(shape, gen) : sweep_blocks_per_sm<double>(shape, false);
@@ -377,11 +381,10 @@ int direct_setup(sbiem_s* s, DevFault<R>& f) {
 // streamed form); other shapes one CTA per SM; with the four-kernel FFT
 // the full grid.
 void sweep_config(sbiem_s* s) {
-  const bool gen = s->fp32() && s->f32.wtab && s->gen_ds_max > 0.0f;
+  const bool gen = on_chip(s, s->gen_ds_max);
   s->f32.gen_ds_max = gen ? s->gen_ds_max : 0.0f;
-  const bool dgen = direct_gen(s, s->gen_ds_max);
-  s->f32.direct.wtab = dgen ? s->direct_wtab : nullptr;
-  s->f32.direct.pieces = dgen ? s->direct_pieces : 0;
+  s->f32.direct.wtab = gen ? s->direct_wtab : nullptr;
+  s->f32.direct.pieces = gen ? s->direct_pieces : 0;
   int per_sm = sweep_blocks(s, s->sweep_shape, s->gen_ds_max);
   if (s->sweep_ctas > 0 && s->sweep_ctas < per_sm) per_sm = s->sweep_ctas;
   s->hist_grid = s->sm_count * per_sm;
@@ -1049,7 +1052,7 @@ int sbiem_create(sbiem_t* out, const sbiem_params* pin, const double* h, const d
         }
       }
     }
-    if (rc == SBIEM_OK && direct_form(s, 3)) rc = direct_setup<float>(s, s->f32);
+    if (rc == SBIEM_OK && can_direct(s, 3)) rc = direct_setup<float>(s, s->f32);
     sweep_config(s);
   } else {
     f.ring = alloc_n<Slot64>(s, static_cast<size_t>(std::max<int64_t>(s->total_slots, 1)), &ok);
@@ -1763,7 +1766,7 @@ int sbiem_footprint(sbiem_t s, int64_t* hist_bytes, int64_t* device_bytes) {
   // weights stream only for the modes that do not evaluate them on chip
   int64_t streamed = 0;
   // the direct sweep's table serves every mode, or none
-  const bool direct = s->fp32() && direct_form(s, s->sweep_shape);
+  const bool direct = s->fp32() && direct_form(s, s->sweep_shape, s->gen_ds_max);
   const bool none = direct && s->f32.direct.wtab;
   for (int n = 1; n < s->nmodes && !none; ++n) {
     const double ds = s->p.cs * (2.0 * M_PI * n / s->L) * s->dt_min;
@@ -1782,6 +1785,7 @@ int sbiem_set_wait_limit(sbiem_t s, int64_t polls) {
   s->spin_limit = polls;
   s->f64.spin_limit = polls;
   s->f32.spin_limit = polls;
+  sweep_config(s);  // the limit decides between the two forms of the sweep
   drop_graphs(s);
   s->lag_m = -1;
   return SBIEM_OK;
@@ -1795,7 +1799,8 @@ int sbiem_get_sweep(sbiem_t s, int32_t* shape, double* gen_ds_max, int32_t* ctas
   if (ctas_per_sm) *ctas_per_sm = s->hist_grid / (s->sm_count > 0 ? s->sm_count : 1);
   if (lag_ctas_per_sm) *lag_ctas_per_sm = s->lag_grid / (s->sm_count > 0 ? s->sm_count : 1);
   if (table_err)
-    *table_err = s->gen_pieces <= 0 ? -1.0 : (direct_form(s, s->sweep_shape) && s->direct_wtab ? s->direct_err : s->gen_err);
+    *table_err = s->gen_pieces <= 0 ? -1.0
+                 : s->direct_wtab && direct_form(s, s->sweep_shape, s->gen_ds_max) ? s->direct_err : s->gen_err;
   return SBIEM_OK;
 }
 
@@ -1854,7 +1859,7 @@ int sbiem_tune(sbiem_t s, int reps, int32_t* shape_out, double* gen_out, int32_t
     if (sweep_chunk_slots(s->p.precision, shape) != s->chunk_slots) continue;
     for (float t : thr) {
       // the direct sweep's table serves every mode: one threshold stands for all
-      if (direct_form(s, shape) && t > 0.0f && t != kGenDsMaxDefault) continue;
+      if (t > 0.0f && t != kGenDsMaxDefault && direct_form(s, shape, t)) continue;
       const int lim = sweep_blocks(s, shape, t);
       for (int c = 1; c <= lim; ++c) {
         s->sweep_shape = shape;
@@ -2214,14 +2219,18 @@ int batch_use_chunks(sbiem_batch_s* b, int64_t slots) {
   return SBIEM_OK;
 }
 
-// Whether the ensemble's direct sweep takes its weights from the table.
-bool batch_direct_gen(const sbiem_batch_s* b) { return b->fp32 && b->gen && b->direct_wtab; }
+// Whether the ensemble's history launch of this shape and weight form is the
+// direct sweep: shape 3 at every N (the 16-member ensemble's sweep 120 us,
+// bulk-async 279), and with on-chip weights only by a table of its own.
+bool batch_direct_form(const sbiem_batch_s* b, int shape, bool gen) {
+  return shape == 3 && !(b->fp32 && gen && !b->direct_wtab);
+}
 
 // Resident CTAs per SM of the ensemble's history launch in a sweep shape.
 int batch_blocks(const sbiem_batch_s* b, int shape, bool gen) {
   int n;
-  if (shape == 3)
-    n = b->fp32 ? direct_blocks_per_sm<float>(gen && b->direct_wtab, b->direct_pieces, true)
+  if (batch_direct_form(b, shape, gen))
+    n = b->fp32 ? direct_blocks_per_sm<float>(gen, b->direct_pieces, true)
                 : direct_blocks_per_sm<double>(false, 0, true);
   else
     n = b->fp32 ? persist_blocks_per_sm<float>(shape, gen) : persist_blocks_per_sm<double>(shape, false);
@@ -2348,9 +2357,9 @@ void batch_history(sbiem_batch_s* b, cudaStream_t st, bool ahead = false) {
   const bool gen = sizeof(R) == 4 && b->gen;
   const int resident = b->sm_count * batch_blocks(b, b->shape, gen);
   if (grid > resident) grid = resident;
-  if (b->shape == 3) {
+  if (batch_direct_form(b, b->shape, gen)) {
     auto t = batch_direct<R>(b);
-    t.wtab = batch_direct_gen(b) ? b->direct_wtab : nullptr;
+    t.wtab = gen ? b->direct_wtab : nullptr;
     t.pieces = t.wtab ? b->direct_pieces : 0;
     const SweepBarrier bar{b->bar, b->bar + 1, b->bar_limit, static_cast<int>(b->members.size())};
     launch_direct_batch<R>(t, static_cast<const DevFault<R>*>(b->fs), b->direct_partial, ahead ? 2 : 1, grid, ahead,
@@ -2465,19 +2474,24 @@ int sbiem_batch_create(sbiem_batch_t* out, int n, const sbiem_t* members, int64_
   if (fp32) {
     // one weight table for all: the members' tables cover each its own s
     // range of one function when c_s/c_p and dt_min agree; take the widest
-    bool same = true;
-    const sbiem_s* widest = members[0];
+    // (the direct sweep's: when every member has one)
+    bool same = true, direct = true;
+    const sbiem_s *widest = members[0], *dwidest = members[0];
     for (int r = 0; r < n; ++r) {
       const sbiem_s* m = members[r];
-      same = same && m->f32.wtab && (m->direct_wtab != nullptr) == (members[0]->direct_wtab != nullptr) && m->p.cs / m->p.cp == members[0]->p.cs / members[0]->p.cp &&
+      same = same && m->f32.wtab && m->p.cs / m->p.cp == members[0]->p.cs / members[0]->p.cp &&
              m->dt_min == members[0]->dt_min;
+      direct = direct && m->direct_wtab;
       if (m->gen_pieces > widest->gen_pieces) widest = m;
+      if (m->direct_pieces > dwidest->direct_pieces) dwidest = m;
     }
     if (same) {
       b->wtab = widest->f32.wtab;
       b->gen_pieces = widest->gen_pieces;
-      b->direct_wtab = widest->direct_wtab;
-      b->direct_pieces = widest->direct_pieces;
+      if (direct) {
+        b->direct_wtab = dwidest->direct_wtab;
+        b->direct_pieces = dwidest->direct_pieces;
+      }
       b->gen = true;
       b->gen_ds_max = kGenDsMaxDefault;
     }
@@ -2505,7 +2519,7 @@ int sbiem_batch_create(sbiem_batch_t* out, int n, const sbiem_t* members, int64_
     // the overlapped sweep leaves room for the one-launch FP32 passes
     bool small = fp32;
     for (auto* m : b->members) small = small && m->N <= kFusedMaxN;
-    b->lag_grid = small && b->shape != 3 ? b->sm_count : b->hist_grid;
+    b->lag_grid = small && !batch_direct_form(b, b->shape, b->gen) ? b->sm_count : b->hist_grid;
   }
   for (auto* m : b->members) cudaStreamSynchronize(m->stream);
   int rc = fp32 ? batch_build<float>(b) : batch_build<double>(b);
@@ -2660,7 +2674,8 @@ int sbiem_batch_tune(sbiem_batch_t b, int reps, int64_t* chunk_out, int* blocks_
     b->shape = sh;
     b->gen = tv > 0.0f;
     b->gen_ds_max = tv;
-    if (sh == 3 && tv > 0.0f && tv != kGenDsMaxDefault) continue;  // one threshold stands for all
+    // the direct sweep's table serves every mode: one threshold stands for all
+    if (tv > 0.0f && tv != kGenDsMaxDefault && batch_direct_form(b, sh, true)) continue;
     const int lim = batch_blocks(b, sh, b->gen);
     for (int bl = 1; bl <= lim; ++bl) {
       b->hist_grid = b->sm_count * bl;

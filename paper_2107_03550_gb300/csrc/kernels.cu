@@ -1459,7 +1459,7 @@ __global__ void __launch_bounds__(kHistThreads)
 // stages; shape 4: shape 3's chunks in one stage (49 KB), for the sweep that
 // runs beside the spectral passes: two of its CTAs and a pass CTA share an SM.
 // Where the direct sweep (direct.cu) is the better form it takes shape 3's
-// place (use_direct).
+// place (direct_rule).
 template <class R, int SH> struct SweepCfg {
   static constexpr int kBase = sizeof(R) == 4 ? 512 : 256;
   static constexpr int kSlots = SH == 1 ? 2 * kBase : (SH >= 3 ? 4 * kBase : kBase);
@@ -3057,16 +3057,6 @@ static void launch_finish(const DevFault<R>& f, double2* outT, double2* outN, bo
   const DevFault<R> fv = f;
   const int G = sweep_grid(grid, f.nchunks);
   launch_early(k_sweep_finish<R>, dim3((f.nmodes + 255) / 256), dim3(256), 0, st, fv, outT, outN, f32, G);
-}
-
-// Shape 3 is the direct sweep in FP64 and, in FP32, above kFusedMaxN (sweep
-// alone, direct against bulk-async: FP64 N = 1024 12.5 and 24.9 us, 8192 68
-// and 129 us, 65536 513 and 1210 us; FP32 N = 65536 183 and 222 us, 262144 782
-// and 980 us; at N = 4096 21.0 and 18.5 us).  A caller's own copy-wait limit
-// asks for the form that has such waits.
-template <class R>
-static bool use_direct(const DevFault<R>& f, int shape) {
-  return shape == 3 && (sizeof(R) == 8 || f.N > kFusedMaxN) && f.spin_limit == kSpinLimit;
 }
 
 template <class R>
