@@ -21,8 +21,12 @@
 //
 // Weights (FP32): every mode's weights come from the table, per lag: s = (j +
 // 1/2) ds in units of the piece width as two floats, the nearest piece, a
-// degree-4 polynomial in the offset (table error 4e-9 of max|C|, the rest is
-// rounding: about two roundings of the weight, where a stored weight has one).
+// degree-4 polynomial in the offset, with the constant as two floats so that
+// the weight is rounded once, as a stored one is.  Against 64 bits over all
+// lags (N = 32768 to 262144, k_c L = 120 to 300, r = 0.58): rms 2.59e-8 of the
+// weights' (stored 2.58e-8; with a constant of one float, whose rounding all
+// lags of a piece share, 3.6e-8), largest 4.4e-8 of max|C| (3.8e-8; 7.7e-8);
+// the table itself is within 2.9e-9.
 // About 40 instructions per 32 lags, 43 % of the issue slots, where streaming
 // the weights costs half the ring bytes again (N = 262144: 782 against 1093
 // us).  Degree 5 on pieces twice as wide (one more 128-bit table read per lag;
@@ -104,21 +108,24 @@ __device__ __forceinline__ void direct_fma(Acc64& a, const Slot64& s, const doub
 }
 
 // (w^T, w^N) at lag jf - 1/2 from the table in shared memory (P pieces): dh
-// + dl is ds over the piece width.
+// + dl is ds over the piece width.  The lower part of the constant, its shift
+// out of the top coefficient's word included, is three instructions of about
+// 30: N = 262144 steps 922 -> 926 us, N = 65536 211 -> 212 us.
 __device__ __forceinline__ float2 table_weight(const float4* __restrict__ tab, int P, float jf, float dh, float dl) {
   constexpr float kMagic = 12582912.0f;  // 1.5 * 2^23: adding it rounds to an integer
-  const float p = jf * dh;
-  const float e = fmaf(jf, dl, fmaf(jf, dh, -p));
-  const float g = p + kMagic;
-  const float u = (p - (g - kMagic)) + e;  // the difference is exact
+  const float g = fmaf(jf, dh, kMagic);
+  const float u = fmaf(jf, dl, fmaf(jf, dh, kMagic - g));  // kMagic - g is exact, |u| about 1/2 at most
   const int q = __float_as_int(g) - __float_as_int(kMagic);
   const float4 g0 = tab[q], g1 = tab[P + q];
   const float2 g2 = reinterpret_cast<const float2*>(tab + 2 * P)[q];
   const float2 uu = make_float2(u, u);
+  // g2: the top coefficient, with the lower part of the constant in its lower half
   float2 w = ffma2(g2, uu, make_float2(g1.z, g1.w));
   w = ffma2(w, uu, make_float2(g1.x, g1.y));
   w = ffma2(w, uu, make_float2(g0.z, g0.w));
-  return ffma2(w, uu, make_float2(g0.x, g0.y));
+  w = ffma2(w, uu, make_float2(__uint_as_float(__float_as_uint(g2.x) << 16),
+                               __uint_as_float(__float_as_uint(g2.y) << 16)));
+  return fadd2(w, make_float2(g0.x, g0.y));  // the one rounding of the weight's size
 }
 
 // Float4s of the table: two per piece and a float2.
@@ -256,6 +263,8 @@ __device__ __forceinline__ void direct_items(const DirectItem<R>* __restrict__ i
       li = lend;
     }
     const bool whole = min(jend, min(mt, mn)) - jc >= 32 * U;
+    // the lane's first lag, converted once: lags stay below 2^23, so adding the row and 1/2 is exact
+    const float jl = static_cast<float>(jc + lane);
     typename AccT<R>::T acc{};
     if constexpr (sizeof(R) == 8) acc = run;
 #pragma unroll
@@ -264,7 +273,7 @@ __device__ __forceinline__ void direct_items(const DirectItem<R>* __restrict__ i
 #pragma unroll
         for (int u = g * G; u < g * G + G; ++u) {
           W2<R> w;
-          if constexpr (GEN) w = table_weight(tab, P, static_cast<float>(jc + 32 * u + lane) + 0.5f, dh, dl);
+          if constexpr (GEN) w = table_weight(tab, P, jl + (32.0f * u + 0.5f), dh, dl);
           else w = wv[u];
           direct_fma(acc, v[u], w);
         }
@@ -274,7 +283,7 @@ __device__ __forceinline__ void direct_items(const DirectItem<R>* __restrict__ i
           if (32 * u + lane < jend - jc) {
             const int j = jc + 32 * u + lane;
             W2<R> w;
-            if constexpr (GEN) w = table_weight(tab, P, static_cast<float>(j) + 0.5f, dh, dl);
+            if constexpr (GEN) w = table_weight(tab, P, jl + (32.0f * u + 0.5f), dh, dl);
             else w = wv[u];
             if (j >= mt) w.x = R(0);
             if (j >= mn) w.y = R(0);

@@ -24,6 +24,8 @@
 //   J0, J1 are the C library's j0/j1.
 #include <algorithm>
 #include <cmath>
+#include <cstdint>
+#include <cstring>
 #include <vector>
 
 #include "internal.h"
@@ -312,15 +314,48 @@ void cheb_eval(const ChebTable& c, double s, double* cT, double* cN) {
 }
 }  // namespace
 
+namespace {
+// The interpolating polynomial of v at the n <= 5 points x, to powers of u
+// (Newton's divided differences; v is overwritten).
+void interpolate(int n, const double* x, double* v, double* a) {
+  for (int k = 1; k < n; ++k)
+    for (int i = n - 1; i >= k; --i) v[i] = (v[i] - v[i - 1]) / (x[i] - x[i - k]);
+  for (int i = 0; i < n; ++i) a[i] = 0.0;
+  for (int k = n - 1; k >= 0; --k) {
+    // a <- a (u - x_k) + v_k
+    for (int i = n - 1; i >= 1; --i) a[i] = a[i - 1] - x[k] * a[i];
+    a[0] = v[k] - x[k] * a[0];
+  }
+}
+
+// The upper 16 bits of an FP32 value rounded to 8 significant bits.
+uint32_t upper16(float v) {
+  uint32_t b;
+  std::memcpy(&b, &v, 4);
+  return (b + 0x8000u) >> 16;
+}
+float from_bits(uint32_t b) {
+  float v;
+  std::memcpy(&v, &b, 4);
+  return v;
+}
+}  // namespace
+
 // FP32 table of the weights dt C(s) for the direct sweep.  Piece q is centred
 // at s = q kDirectH and serves |s - q kDirectH| <= kDirectH / 2 (piece 0: s >=
 // 0): a polynomial of degree kDirectDeg in u = s / kDirectH - q, |u| <= 1/2,
-// interpolating at the Chebyshev nodes of that range.  Layout for P pieces:
-// P x (c0T, c0N, c1T, c1N), P x (c2T, c2N, c3T, c3N), P x (c4T, c4N).
+// interpolating at the Chebyshev nodes of that range.  A weight is to be
+// rounded once, as a stored one is, so the constant is kept as two floats, the
+// lower with 8 significant bits: it shares a word with the top coefficient,
+// which is rounded to 8 bits above it and read with those lower bits in place;
+// the others then interpolate what that coefficient leaves (its rounding is
+// 1e-9 of max|C| after that).
+// Layout for P pieces: P x (c0T, c0N, c1T, c1N), P x (c2T, c2N, c3T, c3N), P x
+// (word T, word N), word = upper half c4, lower half the rest of c0.
 // Interpolation error: |C^(5)| (kDirectH / 2)^5 / (5! 2^4), with the kernels
-// oscillating at up to 1/r in s about 5e-9 of max|C|.  *max_err: the largest
-// |table - dt C| over 16 points per piece, evaluated in FP64 from the rounded
-// coefficients, over dt max|C|.
+// oscillating at up to 1/r in s (r = c_s/c_p): 4e-9 of max|C| for r = 0.58,
+// and growing like r^-5.  *max_err: the largest |table - dt C| over 16 points
+// per piece, evaluated in FP64 from the rounded coefficients, over dt max|C|.
 void build_direct_table(const ChebTable& cheb, double dt, double smax, std::vector<float>& tab, int* npieces,
                         double* max_err) {
   constexpr int n = kDirectDeg + 1;
@@ -330,41 +365,46 @@ void build_direct_table(const ChebTable& cheb, double dt, double smax, std::vect
   tab.assign((static_cast<size_t>(2) * P + (P + 1) / 2) * 4, 0.0f);
   double err = 0.0, cmax = 0.0;
   for (int q = 0; q < P; ++q) {
-    // nodes in u: the piece's half of the range where it starts at s = 0
+    // the piece's range of u: half of it where it starts at s = 0
     const double lo = q == 0 ? 0.0 : -0.5, hi = 0.5;
-    double x[n], c[2][n];
-    for (int i = 0; i < n; ++i) {
-      x[i] = 0.5 * (lo + hi) + 0.5 * (hi - lo) * std::cos(M_PI * (i + 0.5) / n);
-      cheb_eval(cheb, (q + x[i]) * kDirectH, &c[0][i], &c[1][i]);
-    }
-    for (int f = 0; f < 2; ++f) {
-      // Newton's divided differences, then to powers of u
-      double d[n];
-      for (int i = 0; i < n; ++i) d[i] = c[f][i];
-      for (int k = 1; k < n; ++k)
-        for (int i = n - 1; i >= k; --i) d[i] = (d[i] - d[i - 1]) / (x[i] - x[i - k]);
-      double a[n] = {0.0};
-      for (int k = n - 1; k >= 0; --k) {
-        // a <- a (u - x_k) + d_k
-        for (int i = n - 1; i >= 1; --i) a[i] = a[i - 1] - x[k] * a[i];
-        a[0] = d[k] - x[k] * a[0];
+    double v[2][n], x[n], a[2][n];
+    // c[f] at the m Chebyshev nodes of the range
+    auto sample = [&](int m) {
+      for (int i = 0; i < m; ++i) {
+        x[i] = 0.5 * (lo + hi) + 0.5 * (hi - lo) * std::cos(M_PI * (i + 0.5) / m);
+        cheb_eval(cheb, (q + x[i]) * kDirectH, &v[0][i], &v[1][i]);
+        v[0][i] *= dt;
+        v[1][i] *= dt;
       }
-      for (int k = 0; k < 4; ++k)
-        tab[4 * (static_cast<size_t>(k / 2) * P + q) + 2 * (k & 1) + f] = static_cast<float>(dt * a[k]);
-      tab[static_cast<size_t>(8) * P + 2 * q + f] = static_cast<float>(dt * a[4]);
+    };
+    sample(n);
+    for (int f = 0; f < 2; ++f) interpolate(n, x, v[f], a[f]);
+    sample(n - 1);
+    for (int f = 0; f < 2; ++f) {
+      const uint32_t top = upper16(static_cast<float>(a[f][4])) << 16;
+      const float c0 = static_cast<float>(a[f][0]);
+      const float c4 = from_bits(top | upper16(static_cast<float>(a[f][0] - c0)));
+      for (int i = 0; i < n - 1; ++i) v[f][i] -= c4 * ((x[i] * x[i]) * (x[i] * x[i]));
+      interpolate(n - 1, x, v[f], a[f]);
+      const uint32_t low = upper16(static_cast<float>(a[f][0] - c0));
+      tab[4 * static_cast<size_t>(q) + f] = c0;
+      for (int k = 1; k < 4; ++k)
+        tab[4 * (static_cast<size_t>(k / 2) * P + q) + 2 * (k & 1) + f] = static_cast<float>(a[f][k]);
+      tab[static_cast<size_t>(8) * P + 2 * q + f] = from_bits(top | low);
+      // what the sweep evaluates
+      a[f][0] = static_cast<double>(c0) + from_bits(low << 16);
+      for (int k = 1; k < 4; ++k) a[f][k] = static_cast<float>(a[f][k]);
+      a[f][4] = from_bits(top | low);
     }
     for (int i = 0; i < 16; ++i) {
       const double u = lo + (hi - lo) * (i + 0.5) / 16.0;
-      double v[2];
-      cheb_eval(cheb, (q + u) * kDirectH, &v[0], &v[1]);
+      double c[2];
+      cheb_eval(cheb, (q + u) * kDirectH, &c[0], &c[1]);
       for (int f = 0; f < 2; ++f) {
-        const size_t P4 = static_cast<size_t>(4) * P;
-        const double a[n] = {tab[4 * q + f], tab[4 * q + 2 + f], tab[P4 + 4 * q + f], tab[P4 + 4 * q + 2 + f],
-                             tab[2 * P4 + 2 * q + f]};
-        double w = a[4];
-        for (int k = 3; k >= 0; --k) w = w * u + a[k];
-        err = std::max(err, std::fabs(w - dt * v[f]));
-        cmax = std::max(cmax, std::fabs(v[f]));
+        double w = a[f][4];
+        for (int k = 3; k >= 0; --k) w = w * u + a[f][k];
+        err = std::max(err, std::fabs(w - dt * c[f]));
+        cmax = std::max(cmax, std::fabs(c[f]));
       }
     }
   }
