@@ -499,8 +499,10 @@ int sbiem_footprint(sbiem_t s, int64_t* history_bytes_per_step, int64_t* device_
  *     16384 and in ensembles shape 3 is the direct sweep instead: one warp
  *     per run of lags, ring slots loaded into registers, no staging in shared
  *     memory and so no copy waits.  A handle with a wait limit of its own
- *     (sbiem_set_wait_limit) sweeps in the bulk-async form; sbiem_get_sweep
- *     and sbiem_footprint report the form in force.
+ *     (sbiem_set_wait_limit) sweeps in the bulk-async form, and so does an
+ *     FP32 handle with on-chip weights whose direct table is off by more than
+ *     1e-8 of max|C| (c_p/c_s above about 2.1); sbiem_get_sweep and
+ *     sbiem_footprint report the form in force.
  *   gen_ds_max (FP32 form only): where the weights come from.  The
  *     midpoint weights w_{n,j} = dt_min C(s) at s = (j + 1/2) ds_n,
  *     ds_n = c_s k_n dt_min, depend on the mode only through ds_n; modes

@@ -1039,16 +1039,21 @@ int sbiem_create(sbiem_t* out, const sbiem_params* pin, const double* h, const d
         s->gen_pieces = gp;
         s->gen_err = gerr;
         s->gen_ds_max = kGenDsMaxDefault;
-        // the direct sweep's table (lags below 2^23 keep (j + 1/2) exact in FP32)
+        // the direct sweep's table (lags below 2^23 keep (j + 1/2) exact in
+        // FP32), where it is as good as stored weights
         if (*std::max_element(s->M.begin(), s->M.end()) < (int64_t(1) << 23)) {
           std::vector<float> dtab;
-          build_direct_table(tab, s->dt_min, smax, dtab, &s->direct_pieces, &s->direct_err);
-          float4* d_dtab = alloc_n<float4>(s, dtab.size() / 4, &ok);
-          if (!ok || up(d_dtab, dtab.data(), sizeof(float) * dtab.size()) != cudaSuccess ||
-              cudaStreamSynchronize(s->stream) != cudaSuccess)
-            rc = nomem(s, "weight table");
-          else
-            s->direct_wtab = d_dtab;
+          int dp = 0;
+          build_direct_table(tab, s->dt_min, smax, dtab, &dp, &s->direct_err);
+          if (s->direct_err <= kDirectTableErr) {
+            s->direct_pieces = dp;
+            float4* d_dtab = alloc_n<float4>(s, dtab.size() / 4, &ok);
+            if (!ok || up(d_dtab, dtab.data(), sizeof(float) * dtab.size()) != cudaSuccess ||
+                cudaStreamSynchronize(s->stream) != cudaSuccess)
+              rc = nomem(s, "weight table");
+            else
+              s->direct_wtab = d_dtab;
+          }
         }
       }
     }
