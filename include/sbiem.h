@@ -467,12 +467,13 @@ int sbiem_harvest_read(sbiem_t s, float* rows_out, int64_t max_rows, int64_t* ro
 int sbiem_mlp_predict(const float* params, const float* X, int64_t n, float* out);
 /* Mean-squared-error loss over normalized inputs X[n][5] and targets t[n]
  * and its gradient with respect to the SBIEM_MLP_PARAMS weights (FP32, own
- * forward / backward kernels, fixed-order reduction). */
+ * forward / backward kernels; the order of the sums follows from n alone). */
 int sbiem_mlp_grad(const float* params, const float* X, const float* t, int64_t n, float* grad, float* loss);
 /* Train on n harvested rows (host, 6 floats each): normalization from the
  * data, seeded initialization, Adam (lr) on shuffled batches for `epochs`
  * passes, all on the GPU; writes SBIEM_MLP_PARAMS + SBIEM_MLP_NORM values
- * to params and the last batch's loss to *final_loss. */
+ * to params and the last batch's loss to *final_loss.  The order of the sums
+ * follows from n and batch alone, so a seed gives one network. */
 int sbiem_mlp_train(const float* samples, int64_t n, int epochs, int batch, float lr, uint64_t seed,
                     float* params, float* final_loss);
 

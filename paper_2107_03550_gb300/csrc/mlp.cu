@@ -327,15 +327,17 @@ __global__ void __launch_bounds__(256)
 }
 constexpr int kReduceCtas = (kMlpParams + 31) / 32;
 
-// CTAs of k_mlp_grad for B rows: as many as stay resident, one tile at least.
+// CTAs of k_mlp_grad for B rows: one a tile up to two on each of a GB300's 152
+// SMs, all that are resident there.  Each leaves a partial gradient, so their
+// number sets the order of the sums: it follows from the rows alone, not from
+// the SMs that a device or a partition of it offers.
+constexpr int kTrainCtas = 304;
 int train_ctas(int64_t B) {
-  int dev = 0, sms = 0, per = 0;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  cudaFuncSetAttribute(k_mlp_grad, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(sizeof(TrainSmem)));
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_mlp_grad, kTrainThreads, sizeof(TrainSmem));
-  return static_cast<int>(std::max<int64_t>(
-      1, std::min<int64_t>((B + kTileRows - 1) / kTileRows, static_cast<int64_t>(sms) * std::max(per, 1))));
+  return static_cast<int>(std::max<int64_t>(1, std::min<int64_t>((B + kTileRows - 1) / kTileRows, kTrainCtas)));
+}
+cudaError_t configure_train() {
+  return cudaFuncSetAttribute(k_mlp_grad, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              static_cast<int>(sizeof(TrainSmem)));
 }
 
 }  // namespace sbiem
@@ -400,6 +402,7 @@ int sbiem_mlp_grad(const float* params, const float* X, const float* t, int64_t 
   MCK(cudaMemcpy(dp, params, sizeof(float) * kMlpParams, cudaMemcpyHostToDevice));
   MCK(cudaMemcpy(dX, X, sizeof(float) * kMlpIn * n, cudaMemcpyHostToDevice));
   MCK(cudaMemcpy(dt, t, sizeof(float) * n, cudaMemcpyHostToDevice));
+  MCK(configure_train());
   k_mlp_grad<<<nblk, kTrainThreads, sizeof(TrainSmem)>>>(dp, dX, dt, nullptr, 0, static_cast<int>(n), part, lp);
   k_mlp_reduce<<<kReduceCtas, 256>>>(part, nblk, dg, nullptr, nullptr, nullptr, 0.f, 0.f, 0.f, 0.f, 0);
   MCK(cudaGetLastError());
@@ -477,6 +480,7 @@ int sbiem_mlp_train(const float* samples, int64_t n, int epochs, int batch, floa
   MCK(cudaMemset(m2, 0, sizeof(float) * kMlpParams));
   MCK(cudaMemcpy(dX, Xn.data(), sizeof(float) * kMlpIn * n, cudaMemcpyHostToDevice));
   MCK(cudaMemcpy(dt, tn.data(), sizeof(float) * n, cudaMemcpyHostToDevice));
+  MCK(configure_train());
   for (int ep = 0; ep < epochs; ++ep) {
     std::shuffle(perm.begin(), perm.end(), rng);
     MCK(cudaMemcpy(didx, perm.data(), sizeof(int) * n, cudaMemcpyHostToDevice));
