@@ -305,9 +305,9 @@ def _peaks():
         return 6800.0, "fallback"
 
 
-def _direct(N: int, precision: str) -> bool:
-    """Whether the library's default sweep of such a handle is the direct one (direct.cu)."""
-    return precision == "fp64" or N > 16384
+def _direct(N: int, precision: str, shape: int = 3) -> bool:
+    """Whether the library sweeps such a handle in the direct form (direct.cu) at this shape."""
+    return shape == 3 and (precision == "fp64" or N > 16384)
 
 
 def _direct_source() -> str:
@@ -784,7 +784,8 @@ def run_ours(a):
                        "device_bytes_limit": 180e9,
                        "newton_iters_last_step": {"sum": main["it_sum"], "max": main["it_max"]},
                        "history_ms_with_finish": main["hist_ms"], "sweep": main["sweep"], "side": side},
-            "roofline": {"bound": "hbm", "kernel": "k_direct" if _direct(a.N, a.precision) else "k_sweep",
+            "roofline": {"bound": "hbm",
+                         "kernel": "k_direct" if _direct(a.N, a.precision, main["sweep"]["shape"]) else "k_sweep",
                          "achieved": achieved, "peak": peak,
                          "peak_kind": "measured (MEASURED_PEAKS.json hbm_gbs, burst: the sweep is timed alone)"
                          if peak_kind == "measured" else "fallback 6800 GB/s", "unit": "GB/s",

@@ -378,8 +378,9 @@ int direct_setup(sbiem_s* s, DevFault<R>& f) {
 // chunks (shapes 3 and 4) shape 4 (one stage) on two CTAs per SM (with two
 // stages only one fits beside a pass CTA; flushed N = 4096 steps: 48-50 us
 // with one CTA per SM of the on-chip weight form, 41 us with two of the
-// streamed form); other shapes one CTA per SM; with the four-kernel FFT
-// the full grid.
+// streamed form); other shapes one CTA per SM.  In FP64 and above
+// kFusedMaxN the overlapped sweep has the full grid of its shape (the direct
+// sweep: one CTA per SM, which leaves the passes room).
 void sweep_config(sbiem_s* s) {
   const bool gen = on_chip(s, s->gen_ds_max);
   s->f32.gen_ds_max = gen ? s->gen_ds_max : 0.0f;
@@ -790,9 +791,7 @@ int sbiem_create(sbiem_t* out, const sbiem_params* pin, const double* h, const d
   s->eta = p.mu / (2.0 * p.cs);
   windows(p, s->L, s->dt_min, s->M, s->MT, s->MN);
   {
-    // bulk-async sweep: chunks of one stage buffer (512 lags FP32, 256 FP64),
-    // every resident CTA streaming; the overlapped sweep keeps one CTA per SM
-    // so the pass kernels find room beside it
+    // the chunk length of the default shape; grids and forms by sweep_config
     if (s->fp32()) configure_kernels<float>(make_geom(N, sizeof(float2)));
     else configure_kernels<double>(make_geom(N, sizeof(double2)));
     s->sweep_shape = kDefaultSweepShape;
@@ -1894,14 +1893,13 @@ int sbiem_tune(sbiem_t s, int reps, int32_t* shape_out, double* gen_out, int32_t
       }
     }
   }
-  // With the four-kernel passes (FP32, N > kFusedMaxN) the sweep that is
-  // fastest alone need not give the fastest step: at N = 65536 and 262144
-  // two two-stage CTAs per SM (shape 3) leave the passes room beside the
-  // next step's sweep (steps 0.271 and 1.113 ms, against 0.292 and 1.150 ms
-  // for four one-stage CTAs, the faster sweep alone).  So the best setting
-  // of each shape is timed over real overlapped steps, each undone after
-  // its timing (state snapshot and the overwritten ring slot restored), and
-  // the fastest step is kept.
+  // Above kFusedMaxN (FP32) the sweep that is fastest alone need not give the
+  // fastest step: what counts is also the room it leaves the passes beside the
+  // next step's sweep (of the bulk-async shapes the faster one alone, four
+  // one-stage CTAs per SM, gave the slower step).  So the best setting of each
+  // shape is timed over real overlapped steps, each undone after its timing
+  // (state snapshot and the overwritten ring slot restored), and the fastest
+  // step is kept.
   if (s->fp32() && s->N > kFusedMaxN && s->nmodes > 0) {
     bool ok = ensure_snapshot(s);
     if (ok && !s->tune_slots) {
@@ -1982,10 +1980,8 @@ int sbiem_tune(sbiem_t s, int reps, int32_t* shape_out, double* gen_out, int32_t
   // together for 1 .. (occupancy limit) sweep CTAs per SM; nothing is
   // committed, and the status word the passes may set is put back.  Only
   // where the passes are one-launch kernels that fit beside the sweep (FP32,
-  // N <= kFusedMaxN): with the four-kernel passes the full grid is best (per
-  // step, 3 against 4 CTAs per SM: 1.34 against 1.15 ms at N = 262144, 0.31
-  // against 0.27-0.29 ms at N = 65536), and this proxy, which leaves out the
-  // commit and the graph, picked 3 at N = 65536.
+  // N <= kFusedMaxN); above that the step itself was timed, and the direct
+  // sweep has one CTA per SM.
   if (s->fp32() && s->N <= kFusedMaxN) {
     unsigned st0 = 0;
     CK(cudaMemcpyAsync(&st0, s->f64.status, sizeof(unsigned), cudaMemcpyDeviceToHost, s->stream));
@@ -1995,9 +1991,7 @@ int sbiem_tune(sbiem_t s, int reps, int32_t* shape_out, double* gen_out, int32_t
     const int lim = sweep_blocks(s, s->lag_shape, s->gen_ds_max);
     float lbest = 1e30f;
     int lb = 0;
-    // nine timed launches at least: the candidates' totals are close (with
-    // five, the N = 65536 rough cycle's step came out at 0.27 or 0.31 ms
-    // from run to run)
+    // nine timed launches at least: the candidates' totals are close
     const int reps_lag = std::max(reps, 9);
     for (int c = 1; c <= lim; ++c) {
       s->lag_ctas = c;
@@ -2109,7 +2103,8 @@ struct sbiem_batch_s {
   unsigned* bar = nullptr;
   long long bar_limit = SBIEM_WAIT_LIMIT_DEFAULT;
   // members whose weights are equal read one copy of them (the first such
-  // member's); with any shared the sweep copies ring slots evict-first
+  // member's); with any shared the bulk-async sweep copies ring slots
+  // evict-first
   int distinct_weights = 0;
   bool shared_weights = false;
   bool persistent = true;  // one cooperative launch; false: sweep launch + sum launch
@@ -2723,8 +2718,8 @@ int sbiem_batch_tune(sbiem_batch_t b, int reps, int64_t* chunk_out, int* blocks_
   // The history form (one persistent launch or two launches; they agree
   // bitwise) and the overlap are chosen together: the cooperative launch
   // waits for room beside the passes, so which form is faster depends on the
-  // overlap (256 members: 2.66 ms per step persistent without overlap, 2.42
-  // ms two-launch with it).  Candidates: each form without overlap (its
+  // overlap (256 members with the bulk-async sweep: 2.66 ms per step persistent
+  // without overlap, 2.42 ms two-launch with it).  Candidates: each form without overlap (its
   // sweep alone + the passes) and each form with overlap (its next-step
   // sweep and the passes timed together, for 1 .. (occupancy limit) sweep
   // CTAs per SM).  The passes write only staging arrays, so timing them

@@ -9,7 +9,7 @@
 // (DirectItem, one 64-byte record that holds every static quantity the warp
 // needs).  One warp takes one item at a time, items handed out in strides of
 // the whole grid, so neighbouring items (of like length) run side by side on
-// different SMs and the last round is short.  A warp loads kRows rows of 32
+// different SMs and the last round is short.  A warp loads direct_rows() rows of 32
 // slots into registers with independent 128-bit (FP64: 256-bit) loads, then
 // forms their products; the record and the ring head of its next item are
 // brought into L1 ahead.  Nothing is
@@ -374,8 +374,7 @@ __device__ __forceinline__ double sum_items(const double* partial, int first, in
   return warp_reduce4<double>(a.x, a.y, a.z, a.w);
 }
 
-// Modes of several items (fc[t] = (mode, first item), their counts in cnt):
-// one warp each.
+// Modes of several items (runs[t]: mode, first item, count): one warp each.
 template <class R>
 __global__ void __launch_bounds__(kFinishThreads)
     k_direct_finish(const DirectRun* __restrict__ runs, int nruns, const double* partial, double2* outT, double2* outN,

@@ -1,11 +1,16 @@
 // sm_103a kernels of the non-planar spectral BIEM time step (Sec. 3.3).
 //
-//   k_history  truncated history convolution A^X_n = sum_j w^X_{n,j} H^X_n
-//              (Sec. 3.1, Sec. 3.3 step (2)), the bandwidth-bound hot loop
-//   k_col      column pass of the four-step FFT; forward with the predictor
-//              prologue (Vbar, kappa Vbar), inverse with the spectral
-//              assembly prologue (static + current-interval + history terms)
-//   k_row      row pass of the four-step FFT
+//   k_sweep    truncated history convolution A^X_n = sum_j w^X_{n,j} H^X_n
+//              (Sec. 3.1, Sec. 3.3 step (2)) in its bulk-async form (the
+//              direct form: direct.cu)
+//   k_spectral_fused, k_spectral_cluster, k_spectral_cluster64
+//              one-launch spectral pass: forward FFT of (Vbar, kappa Vbar),
+//              assembly (static + current-interval + history terms), inverse
+//   k_pass_col, k_pass_mid, k_pass_row
+//              the FP32 pass above N = 16384
+//   k_col, k_row
+//              the FP64 pass above N = 8192: columns (with the predictor or
+//              the assembly ahead of the transform) and rows, each direction
 //   k_newton   per-element state update and Newton solve of Eq. (momentum)
 //              with radiation damping (Sec. 3.3 step (3))
 //   k_commit   accept the step: state, spectral running sums, history push
@@ -41,8 +46,9 @@ template <class C> __device__ __forceinline__ C cmul(C a, C b) {
 // then writes, so one buffer suffices.
 constexpr int kMaxBfly = 8;
 
-template <class C, bool INV>
-__device__ void fft_batch(C* buf, int lgM, int B, const C* twm, int tid, int nth) {
+template <bool INV>
+__device__ void fft_batch(double2* buf, int lgM, int B, const double2* twm, int tid, int nth) {
+  using C = double2;
   const int M = 1 << lgM;
   const int half = M >> 1;
   const int total = B * half;
@@ -93,17 +99,16 @@ enum { PRO_LOAD = 0, PRO_PASS = 1, PRO_ASSEMBLE = 2 };
 //   tau_m = -|k| [ S (Dhat + dt U) + mu (w0T U + AT) ]
 //   sig_m = -i sgn(k) [ S (Khat + dt Q) + mu (w0N Q + AN) ]   (0 at m = 0, N/2)
 // and Y_n = tau_n + i sig_n of the full spectrum (conjugates for n > N/2).
-template <class R>
-__device__ __forceinline__ Cx<R> assemble(const DevFault<R>& f, int n, int pass, int m_dt, double dt) {
+__device__ __forceinline__ double2 assemble(const DevFault<double>& f, int n, int pass, int m_dt, double dt) {
   const int N = f.N;
   const int m = n <= (N >> 1) ? n : N - n;
-  const Cx<R> Zm = f.Z[m];
-  const Cx<R> Zc = f.Z[(N - m) & (N - 1)];
+  const double2 Zm = f.Z[m];
+  const double2 Zc = f.Z[(N - m) & (N - 1)];
   double2 U, Q;
-  U.x = 0.5 * (static_cast<double>(Zm.x) + static_cast<double>(Zc.x));
-  U.y = 0.5 * (static_cast<double>(Zm.y) - static_cast<double>(Zc.y));
-  Q.x = 0.5 * (static_cast<double>(Zm.y) + static_cast<double>(Zc.y));
-  Q.y = -0.5 * (static_cast<double>(Zm.x) - static_cast<double>(Zc.x));
+  U.x = 0.5 * (Zm.x + Zc.x);
+  U.y = 0.5 * (Zm.y - Zc.y);
+  Q.x = 0.5 * (Zm.y + Zc.y);
+  Q.y = -0.5 * (Zm.x - Zc.x);
   double tr = 0.0, ti = 0.0, sr = 0.0, si = 0.0;
   if (m > 0) {
     const double k = kTwoPi * m / f.L;
@@ -117,9 +122,9 @@ __device__ __forceinline__ Cx<R> assemble(const DevFault<R>& f, int n, int pass,
       const int lim = min(m_dt, f.Mn[m]);
       const int64_t wo = f.w_off[m];
       for (int j = 0; j < lim; ++j) {
-        const W2<R> w = f.w[wo + j];
-        w0T += static_cast<double>(w.x);
-        w0N += static_cast<double>(w.y);
+        const double2 w = f.w[wo + j];
+        w0T += w.x;
+        w0N += w.y;
       }
     }
     const double2 D = f.dhat[m], K = f.khat[m], AT = f.AT[m], AN = f.AN[m];
@@ -145,10 +150,7 @@ __device__ __forceinline__ Cx<R> assemble(const DevFault<R>& f, int n, int pass,
     ti = -ti;
     si = -si;
   }
-  Cx<R> Y;
-  Y.x = static_cast<R>(tr - si);
-  Y.y = static_cast<R>(ti + sr);
-  return Y;
+  return make_double2(tr - si, ti + sr);
 }
 
 // Per-mode inputs of the precision form's assembly: running sums F[delta],
@@ -275,11 +277,11 @@ __device__ __forceinline__ void reset_newton_stats(const DevFault<R>& f, int pas
   }
 }
 
-template <class R, bool INV, int PRO>
-__device__ __forceinline__ void col_body(const FftGeom& g, const Cx<R>* __restrict__ tw,
-                                         const Cx<R>* __restrict__ in, Cx<R>* __restrict__ out,
-                                         const DevFault<R>& f, int pass, int m_dt, double dt) {
-  using C = Cx<R>;
+template <bool INV, int PRO>
+__device__ __forceinline__ void col_body(const FftGeom& g, const double2* __restrict__ tw,
+                                         const double2* __restrict__ in, double2* __restrict__ out,
+                                         const DevFault<double>& f, int pass, int m_dt, double dt) {
+  using C = double2;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   C* buf = reinterpret_cast<C*>(smem_raw);
   const int M = g.N2, B = g.Bc;
@@ -301,15 +303,15 @@ __device__ __forceinline__ void col_body(const FftGeom& g, const Cx<R>* __restri
     } else if (PRO == PRO_PASS) {
       // predictor slip rate of this pass (Sec. 3.3): V, then (V + V1)/2
       const double vb = (pass == 1) ? f.V[n] : 0.5 * (f.V[n] + f.V1[n]);
-      v.x = static_cast<R>(vb);
-      v.y = static_cast<R>(f.kappa[n] * vb);
+      v.x = vb;
+      v.y = f.kappa[n] * vb;
     } else {
-      v = assemble<R>(f, n, pass, m_dt, dt);
+      v = assemble(f, n, pass, m_dt, dt);
     }
     buf[b * M + n2] = v;
   }
   __syncthreads();
-  fft_batch<C, INV>(buf, g.lgN2, B, twm, tid, nth);
+  fft_batch<INV>(buf, g.lgN2, B, twm, tid, nth);
   for (int t = tid; t < B * M; t += nth) {
     const int b = t % B;
     const int k2 = t / B;
@@ -320,18 +322,18 @@ __device__ __forceinline__ void col_body(const FftGeom& g, const Cx<R>* __restri
   }
 }
 
-template <class R, bool INV, int PRO>
-__global__ void k_col(const FftGeom g, const Cx<R>* __restrict__ tw, const Cx<R>* __restrict__ in,
-                      Cx<R>* __restrict__ out, const __grid_constant__ DevFault<R> f, int pass, int m_dt,
+template <bool INV, int PRO>
+__global__ void k_col(const FftGeom g, const double2* __restrict__ tw, const double2* __restrict__ in,
+                      double2* __restrict__ out, const __grid_constant__ DevFault<double> f, int pass, int m_dt,
                       double dt) {
-  col_body<R, INV, PRO>(g, tw, in, out, f, pass, m_dt, dt);
+  col_body<INV, PRO>(g, tw, in, out, f, pass, m_dt, dt);
 }
 
 // Batched column pass: member blockIdx.y of an ensemble of equal-N faults.
-template <class R, bool INV, int PRO>
-__global__ void k_col_b(const FftGeom g, const DevFault<R>* __restrict__ fs, int pass, int m_dt) {
-  const DevFault<R>& f = fs[blockIdx.y];
-  col_body<R, INV, PRO>(g, f.tw, nullptr, f.zt, f, pass, m_dt, m_dt * f.dt_min);
+template <bool INV, int PRO>
+__global__ void k_col_b(const FftGeom g, const DevFault<double>* __restrict__ fs, int pass, int m_dt) {
+  const DevFault<double>& f = fs[blockIdx.y];
+  col_body<INV, PRO>(g, f.tw, nullptr, f.zt, f, pass, m_dt, m_dt * f.dt_min);
 }
 
 // ------------------------------------------------ FP32 single-CTA spectral pass
@@ -458,44 +460,44 @@ __device__ __forceinline__ void stockham_stage(C* buf, const C* tw, int lgNs, in
   C v[EPT];
   if (!MASK || on) {
 #pragma unroll
-  for (int q = 0; q < NB; ++q) {
-    const int j = tid + q * nth;
-    const int k = j & (Ns - 1);
-    const int tstep = k << (LGL - lgNs - LGR);
+    for (int q = 0; q < NB; ++q) {
+      const int j = tid + q * nth;
+      const int k = j & (Ns - 1);
+      const int tstep = k << (LGL - lgNs - LGR);
 #pragma unroll
-    for (int r = 0; r < R; ++r) {
-      C x = buf[j + r * stride];
-      if (r > 0) {
-        const int a = r * tstep;
-        C w;
-        if constexpr (sizeof(S) == 4) w = a < half ? tw[a] : make_float2(-tw[a - half].x, -tw[a - half].y);
-        else w = tw_full(tw, a, half, false);
-        w.y = flip(w.y, sg);
-        x = f2mul(x, w);
+      for (int r = 0; r < R; ++r) {
+        C x = buf[j + r * stride];
+        if (r > 0) {
+          const int a = r * tstep;
+          C w;
+          if constexpr (sizeof(S) == 4) w = a < half ? tw[a] : make_float2(-tw[a - half].x, -tw[a - half].y);
+          else w = tw_full(tw, a, half, false);
+          w.y = flip(w.y, sg);
+          x = f2mul(x, w);
+        }
+        v[q * R + r] = x;
       }
-      v[q * R + r] = x;
     }
-  }
-  if constexpr (R == 8) {
-    dft8(v, sg);
-  } else if constexpr (R == 4) {
-    dft4<0>(v, sg);
-    if constexpr (EPT == 8) dft4<4>(v, sg);
-  } else {
+    if constexpr (R == 8) {
+      dft8(v, sg);
+    } else if constexpr (R == 4) {
+      dft4<0>(v, sg);
+      if constexpr (EPT == 8) dft4<4>(v, sg);
+    } else {
 #pragma unroll
-    for (int q = 0; q < EPT / 2; ++q) bfly<0>(v[2 * q], v[2 * q + 1], sg);
-  }
+      for (int q = 0; q < EPT / 2; ++q) bfly<0>(v[2 * q], v[2 * q + 1], sg);
+    }
   }
   __syncthreads();
   if (!MASK || on) {
 #pragma unroll
-  for (int q = 0; q < NB; ++q) {
-    const int j = tid + q * nth;
-    const int k = j & (Ns - 1);
-    const int base = ((j - k) << LGR) + k;
+    for (int q = 0; q < NB; ++q) {
+      const int j = tid + q * nth;
+      const int k = j & (Ns - 1);
+      const int base = ((j - k) << LGR) + k;
 #pragma unroll
-    for (int r = 0; r < R; ++r) buf[base + r * Ns] = v[q * R + r];
-  }
+      for (int r = 0; r < R; ++r) buf[base + r * Ns] = v[q * R + r];
+    }
   }
   __syncthreads();
 }
@@ -937,11 +939,11 @@ __global__ void __launch_bounds__(cluster64_threads(1 << LGN))
 
 // Row pass: for k2 in this CTA's B rows, transform t[k2 N1 + n1] over n1
 // (length N1) and store to out[k2 + N2 k1], times scale.
-template <class R, bool INV>
-__device__ __forceinline__ void row_body(const FftGeom& g, const Cx<R>* __restrict__ tw,
-                                         const Cx<R>* __restrict__ in, Cx<R>* __restrict__ out, R scale,
+template <bool INV>
+__device__ __forceinline__ void row_body(const FftGeom& g, const double2* __restrict__ tw,
+                                         const double2* __restrict__ in, double2* __restrict__ out, double scale,
                                          const unsigned* status) {
-  using C = Cx<R>;
+  using C = double2;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   C* buf = reinterpret_cast<C*>(smem_raw);
   const int M = g.N1, B = g.Br;
@@ -956,7 +958,7 @@ __device__ __forceinline__ void row_body(const FftGeom& g, const Cx<R>* __restri
     buf[b * M + n1] = in[(c0 + b) * g.N1 + n1];
   }
   __syncthreads();
-  fft_batch<C, INV>(buf, g.lgN1, B, twm, tid, nth);
+  fft_batch<INV>(buf, g.lgN1, B, twm, tid, nth);
   for (int t = tid; t < B * M; t += nth) {
     const int b = t % B;
     const int k1 = t / B;
@@ -967,16 +969,16 @@ __device__ __forceinline__ void row_body(const FftGeom& g, const Cx<R>* __restri
   }
 }
 
-template <class R, bool INV>
-__global__ void k_row(const FftGeom g, const Cx<R>* __restrict__ tw, const Cx<R>* __restrict__ in,
-                      Cx<R>* __restrict__ out, R scale, const unsigned* status) {
-  row_body<R, INV>(g, tw, in, out, scale, status);
+template <bool INV>
+__global__ void k_row(const FftGeom g, const double2* __restrict__ tw, const double2* __restrict__ in,
+                      double2* __restrict__ out, double scale, const unsigned* status) {
+  row_body<INV>(g, tw, in, out, scale, status);
 }
 
-template <class R, bool INV>
-__global__ void k_row_b(const FftGeom g, const DevFault<R>* __restrict__ fs) {
-  const DevFault<R>& f = fs[blockIdx.y];
-  row_body<R, INV>(g, f.tw, f.zt, INV ? f.y : f.Z, INV ? R(1.0 / g.N) : R(1), f.status);
+template <bool INV>
+__global__ void k_row_b(const FftGeom g, const DevFault<double>* __restrict__ fs) {
+  const DevFault<double>& f = fs[blockIdx.y];
+  row_body<INV>(g, f.tw, f.zt, INV ? f.y : f.Z, INV ? 1.0 / g.N : 1.0, f.status);
 }
 
 // ------------------------------------------- large passes (three launches)
@@ -2809,10 +2811,8 @@ FftGeom make_geom(int N, int elem_bytes) {
   return g;
 }
 
-template <class R>
-static size_t col_smem(const FftGeom& g) { return (static_cast<size_t>(g.Bc) * g.N2 + g.N2 / 2) * sizeof(Cx<R>); }
-template <class R>
-static size_t row_smem(const FftGeom& g) { return (static_cast<size_t>(g.Br) * g.N1 + g.N1 / 2) * sizeof(Cx<R>); }
+static size_t col_smem(const FftGeom& g) { return (static_cast<size_t>(g.Bc) * g.N2 + g.N2 / 2) * sizeof(double2); }
+static size_t row_smem(const FftGeom& g) { return (static_cast<size_t>(g.Br) * g.N1 + g.N1 / 2) * sizeof(double2); }
 
 // Opt in to dynamic shared memory.  The attribute belongs to the function,
 // not to a handle, and handles of different N launch the same kernels, so it
@@ -2926,8 +2926,8 @@ static void launch_early(void (*kernel)(Args...), dim3 grid, dim3 block, size_t 
   launch_attr(kernel, grid, block, smem, st, 1, true, static_cast<cudaEvent_t>(nullptr), args...);
 }
 
-// The spectral part of a pass (forward FFT, assembly, inverse FFT of Sec. 3.3 step (2); the predictor in the
-// FP64 four-kernel form): one launch, or the four-step kernels.
+// The spectral part of a pass (forward FFT, assembly, inverse FFT of Sec. 3.3 step (2)): one launch up to
+// kFusedMaxN (FP32) or kCluster64MaxN (FP64), above them three launches in FP32 and four in FP64.
 template <class R>
 void launch_spectral(const DevFault<R>& f, int pass, int m_dt, cudaStream_t st, cudaEvent_t started) {
   const FftGeom& g = f.g;
@@ -2970,16 +2970,16 @@ void launch_spectral(const DevFault<R>& f, int pass, int m_dt, cudaStream_t st, 
       k_pass_row<L1, L2><<<G::N2 / G::Br, G::trow, 0, st>>>(f);
     });
   } else {
-    const size_t cs = col_smem<R>(g), rs = row_smem<R>(g);
-    auto kfa = k_col<R, false, PRO_PASS>;
-    auto kfb = k_row<R, false>;
-    auto kia = k_col<R, true, PRO_ASSEMBLE>;
-    auto kib = k_row<R, true>;
-    launch_attr(kfa, dim3(g.N1 / g.Bc), dim3(g.tc), cs, st, 1, false, started, g, static_cast<const Cx<R>*>(f.tw),
-                static_cast<const Cx<R>*>(nullptr), f.zt, f, pass, m_dt, dt);
-    kfb<<<g.N2 / g.Br, g.tr, rs, st>>>(g, f.tw, f.zt, f.Z, R(1), f.status);
+    const size_t cs = col_smem(g), rs = row_smem(g);
+    auto kfa = k_col<false, PRO_PASS>;
+    auto kfb = k_row<false>;
+    auto kia = k_col<true, PRO_ASSEMBLE>;
+    auto kib = k_row<true>;
+    launch_attr(kfa, dim3(g.N1 / g.Bc), dim3(g.tc), cs, st, 1, false, started, g, f.tw,
+                static_cast<const double2*>(nullptr), f.zt, f, pass, m_dt, dt);
+    kfb<<<g.N2 / g.Br, g.tr, rs, st>>>(g, f.tw, f.zt, f.Z, 1.0, f.status);
     kia<<<g.N1 / g.Bc, g.tc, cs, st>>>(g, f.tw, nullptr, f.zt, f, pass, m_dt, dt);
-    kib<<<g.N2 / g.Br, g.tr, rs, st>>>(g, f.tw, f.zt, f.y, R(1.0 / g.N), f.status);
+    kib<<<g.N2 / g.Br, g.tr, rs, st>>>(g, f.tw, f.zt, f.y, 1.0 / g.N, f.status);
   }
 }
 
@@ -3216,12 +3216,12 @@ void launch_pass_batch(const FftGeom& g, const DevFault<R>* fs, int members, int
       k_pass_row_b<L1, L2><<<dim3(G::N2 / G::Br, members), G::trow, 0, st>>>(fs);
     });
   } else {
-    const size_t cs = col_smem<R>(g), rs = row_smem<R>(g);
+    const size_t cs = col_smem(g), rs = row_smem(g);
     const dim3 gc(g.N1 / g.Bc, members), gr(g.N2 / g.Br, members);
-    k_col_b<R, false, PRO_PASS><<<gc, g.tc, cs, st>>>(g, fs, pass, m_dt);
-    k_row_b<R, false><<<gr, g.tr, rs, st>>>(g, fs);
-    k_col_b<R, true, PRO_ASSEMBLE><<<gc, g.tc, cs, st>>>(g, fs, pass, m_dt);
-    k_row_b<R, true><<<gr, g.tr, rs, st>>>(g, fs);
+    k_col_b<false, PRO_PASS><<<gc, g.tc, cs, st>>>(g, fs, pass, m_dt);
+    k_row_b<false><<<gr, g.tr, rs, st>>>(g, fs);
+    k_col_b<true, PRO_ASSEMBLE><<<gc, g.tc, cs, st>>>(g, fs, pass, m_dt);
+    k_row_b<true><<<gr, g.tr, rs, st>>>(g, fs);
   }
   k_newton_b<R><<<dim3((N + 31) / 32, members), 32, 0, st>>>(fs, pass, m_dt);  // members use 32 per warp
 }
@@ -3257,15 +3257,15 @@ void configure_batch_kernels(const FftGeom& g) {
       });
   }
   if constexpr (sizeof(R) == 4) {
-  with_pass(g.N, [&](auto l1, auto l2) {
-    constexpr int L1 = decltype(l1)::value, L2 = decltype(l2)::value;
-    allow_smem(k_pass_mid_b<L1, L2>, pass_mid_smem<L1, L2>());
-  });
+    with_pass(g.N, [&](auto l1, auto l2) {
+      constexpr int L1 = decltype(l1)::value, L2 = decltype(l2)::value;
+      allow_smem(k_pass_mid_b<L1, L2>, pass_mid_smem<L1, L2>());
+    });
   } else {
-  allow_smem(k_col_b<R, false, PRO_PASS>, col_smem<R>(g));
-  allow_smem(k_col_b<R, true, PRO_ASSEMBLE>, col_smem<R>(g));
-  allow_smem(k_row_b<R, false>, row_smem<R>(g));
-  allow_smem(k_row_b<R, true>, row_smem<R>(g));
+    allow_smem(k_col_b<false, PRO_PASS>, col_smem(g));
+    allow_smem(k_col_b<true, PRO_ASSEMBLE>, col_smem(g));
+    allow_smem(k_row_b<false>, row_smem(g));
+    allow_smem(k_row_b<true>, row_smem(g));
   }
 }
 
@@ -3387,15 +3387,15 @@ void launch_weights(const DevFault<R>& f, const double* cheb, int npieces, int d
 void launch_fft64(const FftGeom& g, const double2* tw, const double2* in, double2* tmp, double2* out,
                   bool inverse, cudaStream_t st) {
   DevFault<double> none{};
-  const size_t cs = col_smem<double>(g), rs = row_smem<double>(g);
+  const size_t cs = col_smem(g), rs = row_smem(g);
   if (!inverse) {
-    auto kc = k_col<double, false, PRO_LOAD>;
-    auto kr = k_row<double, false>;
+    auto kc = k_col<false, PRO_LOAD>;
+    auto kr = k_row<false>;
     kc<<<g.N1 / g.Bc, g.tc, cs, st>>>(g, tw, in, tmp, none, 0, 0, 0.0);
     kr<<<g.N2 / g.Br, g.tr, rs, st>>>(g, tw, tmp, out, 1.0, nullptr);
   } else {
-    auto kc = k_col<double, true, PRO_LOAD>;
-    auto kr = k_row<double, true>;
+    auto kc = k_col<true, PRO_LOAD>;
+    auto kr = k_row<true>;
     kc<<<g.N1 / g.Bc, g.tc, cs, st>>>(g, tw, in, tmp, none, 0, 0, 0.0);
     kr<<<g.N2 / g.Br, g.tr, rs, st>>>(g, tw, tmp, out, 1.0 / g.N, nullptr);
   }
@@ -3449,26 +3449,23 @@ void configure_kernels(const FftGeom& g) {
         }
       });
   }
-  if constexpr (sizeof(R) == 4) {
-  with_pass(g.N, [&](auto l1, auto l2) {
-    constexpr int L1 = decltype(l1)::value, L2 = decltype(l2)::value;
-    allow_smem(k_pass_mid<L1, L2>, pass_mid_smem<L1, L2>());
-    cudaFuncSetAttribute(k_pass_col<L1, L2>, cudaFuncAttributePreferredSharedMemoryCarveout, kDirectCarveout);
-    cudaFuncSetAttribute(k_pass_mid<L1, L2>, cudaFuncAttributePreferredSharedMemoryCarveout, kDirectCarveout);
-    cudaFuncSetAttribute(k_pass_row<L1, L2>, cudaFuncAttributePreferredSharedMemoryCarveout, kDirectCarveout);
-  });
-  } else {
-  const size_t cs = col_smem<R>(g), rs = row_smem<R>(g);
-  allow_smem(k_col<R, false, PRO_PASS>, cs);
-  allow_smem(k_col<R, true, PRO_ASSEMBLE>, cs);
-  allow_smem(k_row<R, false>, rs);
-  allow_smem(k_row<R, true>, rs);
-  }
   const FftGeom g64 = make_geom(g.N, sizeof(double2));
-  allow_smem(k_col<double, false, PRO_LOAD>, col_smem<double>(g64));
-  allow_smem(k_col<double, true, PRO_LOAD>, col_smem<double>(g64));
-  allow_smem(k_row<double, false>, row_smem<double>(g64));
-  allow_smem(k_row<double, true>, row_smem<double>(g64));
+  if constexpr (sizeof(R) == 4) {
+    with_pass(g.N, [&](auto l1, auto l2) {
+      constexpr int L1 = decltype(l1)::value, L2 = decltype(l2)::value;
+      allow_smem(k_pass_mid<L1, L2>, pass_mid_smem<L1, L2>());
+      cudaFuncSetAttribute(k_pass_col<L1, L2>, cudaFuncAttributePreferredSharedMemoryCarveout, kDirectCarveout);
+      cudaFuncSetAttribute(k_pass_mid<L1, L2>, cudaFuncAttributePreferredSharedMemoryCarveout, kDirectCarveout);
+      cudaFuncSetAttribute(k_pass_row<L1, L2>, cudaFuncAttributePreferredSharedMemoryCarveout, kDirectCarveout);
+    });
+  } else {
+    allow_smem(k_col<false, PRO_PASS>, col_smem(g64));
+    allow_smem(k_col<true, PRO_ASSEMBLE>, col_smem(g64));
+  }
+  allow_smem(k_col<false, PRO_LOAD>, col_smem(g64));
+  allow_smem(k_col<true, PRO_LOAD>, col_smem(g64));
+  allow_smem(k_row<false>, row_smem(g64));
+  allow_smem(k_row<true>, row_smem(g64));
 }
 
 template void launch_history_persist<double>(const DevFault<double>*, const Chunk*, int, double4*, const int2*, int,

@@ -116,7 +116,7 @@ struct DevFault {
   const Chunk* chunks;
   int nchunks;
   const int32_t *mfirst, *mcount;          // per mode: first chunk, chunks
-  int sweep_shape;                         // form of the history sweep (0..4; 3: the direct sweep)
+  int sweep_shape;                         // form of the history sweep (0..4; 3: see direct_rule)
   int lag_shape;                           // the same for the sweep beside the passes (0..4)
   // FP32 sweep with the weights evaluated on chip instead of streamed:
   // per mode (ds_hi, ds_lo, M^T bits, M^N bits) with ds = c_s k_n dt_min as
@@ -149,7 +149,8 @@ struct DevFault {
 
 // One-launch FP32 spectral pass: a single CTA of N/8 threads below
 // kClusterMinN, a cluster of cluster_ctas(N) CTAs from kClusterMinN to
-// kFusedMaxN; larger N use the four-kernel path.
+// kFusedMaxN; larger N take three launches (k_pass_col, k_pass_mid,
+// k_pass_row).
 constexpr int kFusedMaxN = 16384;
 constexpr int kClusterMinN = 2048;
 constexpr int kClusterCTAs = 8;
@@ -166,7 +167,8 @@ constexpr int kCluster64MaxN = 8192;
 __host__ __device__ constexpr int cluster_ctas(int N) { return N >= 4096 ? 16 : kClusterCTAs; }
 // The same for the batched pass of an ensemble (one cluster per member, many
 // clusters at once, beside the overlapped sweep): 8 below N = 16384, where
-// clusters of 16 were slower (256 members: 2.42 against 2.76 ms per step).
+// clusters of 16 were slower (256 members with the bulk-async sweep: 2.42
+// against 2.76 ms per step).
 __host__ __device__ constexpr int batch_cluster_ctas(int N) { return N >= 16384 ? 16 : kClusterCTAs; }
 // Values per thread in each FFT stage of the cluster pass (4: radix-4
 // stages, 8: radix-8 stages with half the threads).
