@@ -27,8 +27,8 @@
 // weights' (stored 2.58e-8; with a constant of one float, whose rounding all
 // lags of a piece share, 3.6e-8), largest 4.4e-8 of max|C| (3.8e-8; 7.7e-8);
 // the table itself is within 2.9e-9.
-// About 40 instructions per 32 lags, 43 % of the issue slots, where streaming
-// the weights costs half the ring bytes again (N = 262144: 782 against 1093
+// About 39 instructions per 32 lags, 38 % of the issue slots, where streaming
+// the weights costs half the ring bytes again (N = 262144: 804 against 1093
 // us).  Degree 5 on pieces twice as wide (one more 128-bit table read per lag;
 // the L1 data path is 70 % busy) took 830 us.
 // FP64, the exact quadrature and windows past the table stream the weights.
@@ -110,7 +110,7 @@ __device__ __forceinline__ void direct_fma(Acc64& a, const Slot64& s, const doub
 // (w^T, w^N) at lag jf - 1/2 from the table in shared memory (P pieces): dh
 // + dl is ds over the piece width.  The lower part of the constant, its shift
 // out of the top coefficient's word included, is three instructions of about
-// 30: N = 262144 steps 922 -> 926 us, N = 65536 211 -> 212 us.
+// 39: N = 262144 steps 922 -> 928 us, N = 65536 211 -> 213 us.
 __device__ __forceinline__ float2 table_weight(const float4* __restrict__ tab, int P, float jf, float dh, float dl) {
   constexpr float kMagic = 12582912.0f;  // 1.5 * 2^23: adding it rounds to an integer
   const float g = fmaf(jf, dh, kMagic);

@@ -198,7 +198,7 @@ template <class R> void configure_direct();
 // Which form a handle's history sweep of a shape takes: shape 3 is the direct
 // sweep in FP64 and, in FP32, above kFusedMaxN (sweep alone, direct against
 // bulk-async: FP64 N = 1024 12.5 and 24.9 us, 8192 68 and 129 us, 65536 513 and
-// 1210 us; FP32 N = 65536 183 and 222 us, 262144 782 and 980 us; at N = 4096
+// 1210 us; FP32 N = 65536 187 and 222 us, 262144 804 and 980 us; at N = 4096
 // 21.0 and 18.5 us).  Two things ask for the bulk-async form: a copy-wait limit
 // of the caller's (only that form has such waits), and on-chip weights (gen)
 // where there is no table of the direct sweep's.
