@@ -311,7 +311,8 @@ int sbiem_history_sums(sbiem_t s, int64_t m, double* AT, double* AN);
  *   mode n), head[n] (int32, ring position of the newest slot of mode n,
  *   0 <= head[n] < R[n], 0 where R[n] = 0; the slot of the i-th newest value
  *   is (head[n] + i) mod R[n]).
- * Outputs: AT, AN (device, nmodes complex FP64 each, re/im interleaved).
+ * Outputs: AT, AN (device, nmodes complex FP64 each, re/im interleaved; 8-byte
+ * aligned).
  * m: the history shift (a step of m dt_min), m >= 1.  stream: cudaStream_t or
  * NULL.
  *

@@ -64,8 +64,8 @@ __device__ __forceinline__ int chunks_of(int32_t r) { return r > 0 ? (r - 1) / k
 // scan took 87 us at 16385 modes, this 6 us.)
 constexpr int kChunkThreads = 1024;
 __global__ void __launch_bounds__(kChunkThreads)
-    k_noalloc_chunks(const int32_t* __restrict__ R, int nmodes, unsigned char* scratch, double2* __restrict__ AT,
-                     double2* __restrict__ AN) {
+    k_noalloc_chunks(const int32_t* __restrict__ R, int nmodes, unsigned char* scratch, double* __restrict__ AT,
+                     double* __restrict__ AN) {
   Header* hd = reinterpret_cast<Header*>(scratch + kOffHeader);
   Chunk* chunks = reinterpret_cast<Chunk*>(scratch + kOffChunks);
   int* counter = reinterpret_cast<int*>(scratch + kOffCounter);
@@ -103,8 +103,9 @@ __global__ void __launch_bounds__(kChunkThreads)
   }
   if (!fits || n >= nmodes) return;
   counter[n] = 0;
-  AT[n] = make_double2(0.0, 0.0);  // modes without history keep this
-  AN[n] = make_double2(0.0, 0.0);
+  // modes without history keep these zeros; 8 bytes a store, which is all the
+  // alignment that a caller's double* has
+  for (double* a : {AT + 2 * n, AN + 2 * n}) a[0] = a[1] = 0.0;
   const int64_t first = c;
   for (int q = 0; q < k; ++q, ++c) {
     Chunk ch;
@@ -138,7 +139,7 @@ int run(int nmodes, int m, const void* ring, const void* weights, const int64_t*
   int rc = setup(&scr);
   if (rc) return rc;
   k_noalloc_chunks<<<(nmodes + kChunkThreads - 1) / kChunkThreads, kChunkThreads, 0, st>>>(
-      Rn, nmodes, scr, reinterpret_cast<double2*>(AT), reinterpret_cast<double2*>(AN));
+      Rn, nmodes, scr, AT, AN);
   if (cudaGetLastError() != cudaSuccess) return SBIEM_ERR_CUDA;
   Header hd;
   if (cudaMemcpyAsync(&hd, scr + kOffHeader, sizeof(hd), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
