@@ -26,7 +26,7 @@
 // lags (N = 32768 to 262144, k_c L = 120 to 300, r = 0.58): rms 2.59e-8 of the
 // weights' (stored 2.58e-8; with a constant of one float, whose rounding all
 // lags of a piece share, 3.6e-8), largest 4.4e-8 of max|C| (3.8e-8; 7.7e-8);
-// the table itself is within 2.9e-9.
+// the table itself is within 4e-9 (2.6 to 3.9e-9 with dt's own rounding).
 // About 39 instructions per 32 lags, 38 % of the issue slots, where streaming
 // the weights costs half the ring bytes again (N = 262144: 804 against 1093
 // us).  Degree 5 on pieces twice as wide (one more 128-bit table read per lag;

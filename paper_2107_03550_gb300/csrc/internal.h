@@ -34,8 +34,8 @@ constexpr double kDirectH = 0.125;
 constexpr int kDirectDeg = 4;
 // Largest error of that table, of dt max|C|, at which it serves: a third of the
 // largest rounding (2^-25) of a stored weight in the binade below max|C|.  The
-// interpolation error grows like (c_p/c_s)^5: 2.9e-9 at c_p/c_s = 1.73, 6.6e-9
-// at 2, 1.1e-8 at 2.2, 7e-8 at 3.
+// interpolation error grows like (c_p/c_s)^5: 2.6 to 3.9e-9 (with dt's own rounding)
+// at c_p/c_s = 1.73, 6.6 to 8.4e-9 at 2, 1.1e-8 at 2.2, 7e-8 at 3.
 constexpr double kDirectTableErr = 1e-8;
 
 void kernel_values(double s, double r, double* cT, double* cN);
